@@ -57,7 +57,10 @@ typedef enum {
 typedef enum { WM_P6 = 0 /* six-hour processor */, WM_P1 = 1 /* one-hour processor */ } wm_processor;
 
 typedef enum {
-  WM_PREC_FP32 = 0,        /* plain path: FP32 FMA everywhere (no TF32), CUDA cores */
+  WM_PREC_FP32 = 0,        /* plain path: FP32 operands, accumulation and results (no TF32). Linear layers on
+                              tensor cores with every operand split exactly into three bf16 parts (error
+                              against float64 no larger than a chain of FP32 FMAs); LayerNorm and attention
+                              in FP32 on CUDA cores */
   WM_PREC_BF16 = 1,        /* BF16 tcgen05 GEMMs + BF16 tensor-core attention, FP32 accumulate,
                               FP32 residual stream, FP32 LayerNorm statistics and softmax normalisers */
   WM_PREC_BF16_FP8MLP = 2  /* as BF16, with the MLP GEMMs in FP8 E4M3 (per-tensor scales) */
@@ -312,7 +315,7 @@ wm_status wm_op_layernorm(const float* x, const float* gamma, const float* beta,
                           int M, int C, float eps, void* stream);
 
 /* Linear layer D = A W^T + bias on A [M, K], W [N, K] (row major, K contiguous).
- * precision WM_PREC_FP32: A, W float32 (CUDA-core FP32 FMA);
+ * precision WM_PREC_FP32: A, W float32 (products exact to 2^-25, FP32 accumulate);
  * precision WM_PREC_BF16: A, W bfloat16 (tcgen05, FP32 accumulate), K % 8 == 0.
  * epilogue 0: out = D (out float32 for FP32, bfloat16 for BF16)
  * epilogue 1: out = GELU(D) (same out types)

@@ -38,6 +38,8 @@ struct BlockW {
   bf16 *fqkv, *f1;
   const float *cs_qkv, *bb_qkv, *cs_1, *bb_1;
   CUtensorMap tm_fqkv[3], tm_f1[3];
+  // FP32: Wqkv, Wo, W1 and W2 split into bf16 planes (k_gemm_f32.cu); NULL until the FP32 path is used
+  bf16 *p_qkv = nullptr, *p_o = nullptr, *p_1 = nullptr, *p_2 = nullptr;
   // FP8 MLP: e4m3 copies of W1, W2 and the static per-tensor scales
   uint8_t *q1, *q2;
   CUtensorMap tm_q1[3], tm_q2[3];
@@ -54,6 +56,8 @@ struct wm_ctx {
   bf16* d_wh = nullptr;
   uint8_t* d_wq = nullptr;   // e4m3 W1, W2 per block
   bf16* d_wf = nullptr;      // LayerNorm-folded bf16 Wqkv, W1 per block
+  bf16* d_wp = nullptr;      // FP32 weights as bf16 planes
+  bool planes_tried = false;
   float2* d_rope_tab = nullptr;       // rotary embedding cos/sin tables (level, latitude, longitude)
   wm::RopeArgs* d_rope = nullptr;     // device copy of rope_host (pointers into d_rope_tab)
   wm::RopeArgs rope_host{};
@@ -151,11 +155,45 @@ void free_workspace(wm_ctx* ctx) {
 
 wm_status tune_block_gemms(wm_ctx* ctx, int batch);
 
+// Once per context, at the FP32 path's first use: every matrix as bf16 planes
+// (six bytes a weight). Without memory for them the GEMMs split W themselves.
+wm_status ensure_planes(wm_ctx* ctx) {
+  if (ctx->planes_tried) return WM_OK;
+  ctx->planes_tried = true;
+  const size_t C = ctx->cfg.C, kc = wm::f32_plane_k((int)C), k4 = wm::f32_plane_k((int)(4 * C));
+  const size_t per = 3 * (8 * C * kc + C * k4);   // Wqkv, Wo, W1 [8C rows of C], W2 [C rows of 4C]
+  const size_t nb = ctx->blk[0].size() + ctx->blk[1].size();
+  if (cudaMalloc(&ctx->d_wp, per * nb * 2) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->d_wp = nullptr;
+    return WM_OK;
+  }
+  bf16* p = ctx->d_wp;
+  for (auto& stack : ctx->blk)
+    for (BlockW& w : stack) {
+      bf16* const q[4] = {p, p + 9 * C * kc, p + 12 * C * kc, p + 24 * C * kc};
+      WM_TRY(wm::launch_split_planes(w.wqkv, q[0], (int)(3 * C), (int)C, 0));
+      WM_TRY(wm::launch_split_planes(w.wo, q[1], (int)C, (int)C, 0));
+      WM_TRY(wm::launch_split_planes(w.w1, q[2], (int)(4 * C), (int)C, 0));
+      WM_TRY(wm::launch_split_planes(w.w2, q[3], (int)C, (int)(4 * C), 0));
+      p += per;
+    }
+  WM_CUDA(cudaDeviceSynchronize());
+  p = ctx->d_wp;
+  for (auto& stack : ctx->blk)
+    for (BlockW& w : stack) {
+      w.p_qkv = p; w.p_o = p + 9 * C * kc; w.p_1 = p + 12 * C * kc; w.p_2 = p + 24 * C * kc;
+      p += per;
+    }
+  return WM_OK;
+}
+
 // Grow the workspace of one precision family to hold `batch` latents. Never
 // called during capture; growing invalidates captured graphs (they hold
 // workspace addresses).
 wm_status ensure_workspace(wm_ctx* ctx, int batch, bool fp32) {
   int& cap = fp32 ? ctx->cap32 : ctx->cap16;
+  if (fp32) WM_TRY(ensure_planes(ctx));
   if (batch <= cap) return WM_OK;
   destroy_graphs(ctx);
   const size_t M = (size_t)batch * ctx->N, C = ctx->cfg.C;
@@ -498,18 +536,18 @@ wm_status block_forward(wm_ctx* ctx, float* x, int batch, int which, int b, bool
     { TimedLaunch t(ctx, WM_K_LN1, s);
       WM_TRY(wm::launch_layernorm(x, w.ln1_g, w.ln1_b, ctx->f_u, false, (int)M, C, c.ln_eps, s)); }
     { TimedLaunch t(ctx, WM_K_QKV, s);
-      WM_TRY(wm::launch_sgemm(ctx->f_u, w.wqkv, w.bqkv, ctx->f_qkv, (int)M, 3 * C, C, wm::EPI_STORE_F32, s));
+      WM_TRY(wm::launch_gemm_f32(ctx->f_u, w.wqkv, w.p_qkv, w.bqkv, ctx->f_qkv, (int)M, 3 * C, C, wm::EPI_STORE_F32, s));
       if (c.rope) WM_TRY(wm::launch_rope_f32(ctx->f_qkv, M, ctx->d_rope, ctx->rope_host, s)); }
     { TimedLaunch t(ctx, WM_K_ATTN, s);
       WM_TRY(wm::launch_na_f32(ctx->f_qkv, ctx->f_o, batch, c.D, c.H, c.W, C, c.heads, c.kd, c.kh, c.kw, per, s)); }
     { TimedLaunch t(ctx, WM_K_PROJ, s);
-      WM_TRY(wm::launch_sgemm(ctx->f_o, w.wo, w.bo, x, (int)M, C, C, wm::EPI_RESID_F32, s)); }
+      WM_TRY(wm::launch_gemm_f32(ctx->f_o, w.wo, w.p_o, w.bo, x, (int)M, C, C, wm::EPI_RESID_F32, s)); }
     { TimedLaunch t(ctx, WM_K_LN2, s);
       WM_TRY(wm::launch_layernorm(x, w.ln2_g, w.ln2_b, ctx->f_u, false, (int)M, C, c.ln_eps, s)); }
     { TimedLaunch t(ctx, WM_K_FC1, s);
-      WM_TRY(wm::launch_sgemm(ctx->f_u, w.w1, w.b1, ctx->f_h, (int)M, 4 * C, C, wm::EPI_GELU, s)); }
+      WM_TRY(wm::launch_gemm_f32(ctx->f_u, w.w1, w.p_1, w.b1, ctx->f_h, (int)M, 4 * C, C, wm::EPI_GELU, s)); }
     { TimedLaunch t(ctx, WM_K_FC2, s);
-      WM_TRY(wm::launch_sgemm(ctx->f_h, w.w2, w.b2, x, (int)M, C, 4 * C, wm::EPI_RESID_F32, s)); }
+      WM_TRY(wm::launch_gemm_f32(ctx->f_h, w.w2, w.p_2, w.b2, x, (int)M, C, 4 * C, wm::EPI_RESID_F32, s)); }
     return WM_OK;
   }
   CUtensorMap tm_x;   // the caller's latent as the residual target
@@ -1102,6 +1140,7 @@ wm_status wm_destroy(wm_ctx* ctx) {
   cudaFree(ctx->d_wh);
   cudaFree(ctx->d_wq);
   cudaFree(ctx->d_wf);
+  cudaFree(ctx->d_wp);
   cudaFree(ctx->d_vf);
   cudaFree(ctx->d_rope_tab);
   cudaFree(ctx->d_rope);
@@ -1500,7 +1539,7 @@ wm_status wm_op_linear(const void* A, const void* W, const float* bias, void* ou
   WM_TRY(wm::prepare_kernels());
   cudaStream_t s = (cudaStream_t)stream;
   if (precision == WM_PREC_FP32)
-    return wm::launch_sgemm((const float*)A, (const float*)W, bias, (float*)out, M, N, K, epilogue, s);
+    return wm::launch_linear_f32((const float*)A, (const float*)W, bias, (float*)out, M, N, K, epilogue, s);
   if (precision != WM_PREC_BF16) return fail(WM_ERR_INVALID_ARG, "linear precision must be FP32 or BF16");
   if (M == 0) return WM_OK;
   if (K % 8 != 0 || N % 8 != 0) return fail(WM_ERR_INVALID_ARG, "BF16 linear needs K % 8 == 0 and N % 8 == 0");

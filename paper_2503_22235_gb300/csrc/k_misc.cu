@@ -57,6 +57,7 @@ int num_sms() {
 }
 
 wm_status prepare_na_f32();
+wm_status prepare_gemm_f32();
 
 wm_status prepare_kernels() {
   static std::mutex mu;
@@ -69,6 +70,7 @@ wm_status prepare_kernels() {
   if (st == WM_OK) st = prepare_na_bf16();
   if (st == WM_OK) st = prepare_na_tc();
   if (st == WM_OK) st = prepare_na_f32();
+  if (st == WM_OK) st = prepare_gemm_f32();
   if (st == WM_OK && !device_status_word()) st = fail(WM_ERR_OOM, "device status word allocation failed");
   if (st == WM_OK && dev >= 0 && dev < 64) done[dev] = true;
   return st;

@@ -211,8 +211,14 @@ wm_status launch_row_stats(const float* x, __nv_bfloat16* xb, float* stats, int 
                            bool pdl = false);
 wm_status launch_layernorm_e4m3(const float* x, const float* g, const float* b, uint8_t* out, int M, int C,
                                 float eps, float inv_scale, cudaStream_t s, bool pdl = false);
-wm_status launch_sgemm(const float* A, const float* W, const float* bias, float* out, int M, int N, int K,
-                       int epi, cudaStream_t s);
+// planes: W split by launch_split_planes (3 N f32_plane_k(K) bf16), or NULL to split it inside the kernel.
+int f32_plane_k(int K);
+wm_status launch_split_planes(const float* W, __nv_bfloat16* planes, int N, int K, cudaStream_t s);
+wm_status launch_gemm_f32(const float* A, const float* W, const __nv_bfloat16* planes, const float* bias, float* out,
+                          int M, int N, int K, int epi, cudaStream_t s);
+// The same for weights met for the first time: splits W for this call where that pays.
+wm_status launch_linear_f32(const float* A, const float* W, const float* bias, float* out, int M, int N, int K,
+                            int epi, cudaStream_t s);
 wm_status launch_na_f32(const float* qkv, float* out, int B, int D, int H, int W, int C, int heads, int kd,
                         int kh, int kw, bool periodic, cudaStream_t s);
 
@@ -241,6 +247,11 @@ bool make_tmap_out(CUtensorMap* map, const void* base, uint64_t rows, uint64_t c
 // the 32-byte swizzle.
 bool make_tmap_e4m3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 bool make_tmap_out_e4m3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols);
+
+// Row-major fp32 [rows, cols]: box 32 columns x box_rows, 128-byte swizzle.
+bool make_tmap_f32(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+// Split weights [3][N][Kp] bf16: box 32 k x box_rows x 3 planes, 64-byte swizzle.
+bool make_tmap_planes(CUtensorMap* map, const void* base, uint64_t N, uint64_t Kp, uint32_t box_rows);
 
 struct GemmArgs {
   CUtensorMap tmA;     // A [M, K], box 128 rows x 128 bytes
