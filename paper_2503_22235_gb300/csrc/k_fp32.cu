@@ -475,6 +475,343 @@ __global__ void __launch_bounds__(256, 2) na_f32_tile_kernel(const float* __rest
     orow[i] = make_float4(o[4 * i] * inv, o[4 * i + 1] * inv, o[4 * i + 2] * inv, o[4 * i + 3] * inv);
 }
 
+// FP32 attention with 2 x 2 blocks of queries (windows of 3, 5 or 7
+// longitudes). A tile of BH x BW blocks of one (batch element, head, level)
+// stages the K and V halo slab of one key level at a time in shared memory
+// (cp.async). TPB threads share a block: each holds the block's four queries
+// and outputs in every TPB-th float4 of the head's channels, so a K or V value
+// read from shared memory serves four queries (196 of the 256 query-key pairs
+// of the block's 8 x 8 keys lie in a 7 x 7 window). A key's four scores are
+// summed over the block's threads by a reduce-scatter (three shuffles at
+// TPB = 4) that leaves each thread the whole score of one query, its own; its
+// probability goes back by three shuffles. A thread keeps the four queries in
+// an order of its own, query (own ^ k) at place k, so neither step selects
+// registers. The block's key rows of a level are divided between the CTA's
+// two halves (the same blocks), whose softmax states are merged at the end.
+// What bounds it (dh = 48, per key of a block and warp): 30 clocks of shared
+// memory (six 128-bit loads of 512 bytes a warp, six shuffles) and 96 of the
+// FMA lanes of one scheduler (48 f32x2, which take two clocks each); 60 % and
+// 53 % busy as measured, three warps a scheduler at 168 registers not hiding
+// all of the loads' and shuffles' latency. 9 x 90 x 180 x 768, 16 heads,
+// window 5 x 7 x 7: 17.2 ms with one query per four threads (every K and V
+// value read for one query only), 4.4 ms here.
+// FP32 FMA and expf throughout. A masked key has probability zero; where its
+// V is not finite that makes the output NaN, and a NaN output is recomputed
+// over its own window alone.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// Four floats from shared memory as two f32x2 operands.
+__device__ __forceinline__ void lds_f2(uint32_t addr, uint64_t& lo, uint64_t& hi) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(a));
+  return f;
+}
+
+// Floats between keys in shared memory: two keys apart lands half the banks
+// away, so that neighbouring blocks' 128-bit loads do not collide.
+template <int DH>
+struct NaBlk {
+  static constexpr int TPB = DH == 64 ? 8 : 4;       // threads per block of queries
+  static constexpr int NI = DH / 4 / TPB;            // float4 per thread
+  static constexpr int KS = DH == 64 ? 64 : DH + 8;
+  static constexpr int MAXT = DH == 48 ? 384 : 512;  // threads per CTA: 168 or 128 registers
+};
+
+// Four channels of one query's output over its own window, in two passes
+// (key0: K of the batch element and head; the channels' V lie C + ch floats on).
+__device__ __noinline__ void na_f32_query(const float* q, const float* key0, float* o, int ch, int H, int W, int C,
+                                          int dh, int ld0, int kd, int r0, int kh, int c0, int kw, float scale) {
+  float mx = -INFINITY, sum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int pass = 0; pass < 2; ++pass)
+    for (int l = 0; l < kd; ++l)
+      for (int r = 0; r < kh; ++r)
+        for (int c = 0; c < kw; ++c) {
+          int lon = c0 + c;
+          while (lon < 0) lon += W;
+          while (lon >= W) lon -= W;
+          const float* key = key0 + (((long)(ld0 + l) * H + r0 + r) * W + lon) * 3 * C;
+          float sc = 0.f;
+          for (int e = 0; e < dh; ++e) sc = fmaf(q[e], key[e], sc);
+          sc *= scale;
+          if (pass == 0) {
+            mx = fmaxf(mx, sc);
+          } else {
+            const float p = expf(sc - mx);
+            sum += p;
+            for (int e = 0; e < 4; ++e) acc[e] = fmaf(p, key[C + ch + e], acc[e]);
+          }
+        }
+  for (int e = 0; e < 4; ++e) o[ch + e] = acc[e] / sum;
+}
+
+template <int DH, int KW>
+__global__ void __launch_bounds__(NaBlk<DH>::MAXT, 1)
+    na_f32_block_kernel(const float* __restrict__ qkv, float* __restrict__ out, int D, int H, int W, int C, int heads,
+                        int kd, int kh, int periodic, int BH, int BW, int tiles_h, int tiles_w,
+                        int* __restrict__ dstatus) {
+  using NB = NaBlk<DH>;
+  constexpr int TPB = NB::TPB, NI = NB::NI, KS = NB::KS, NC = KW + 1, NU = DH / 4;
+  extern __shared__ __align__(16) float sm[];
+  const int HR = min(2 * BH + kh - 1, H);
+  const int WC = periodic ? 2 * BW + KW - 1 : min(2 * BW + KW - 1, W);
+  const int vs = HR * WC * KS;   // K, then V, then one more key: a block may read a column past its window
+  if (threadIdx.x < KS) sm[2 * vs + threadIdx.x] = 0.f;
+  int t = blockIdx.x;
+  const int tw = t % tiles_w;
+  t /= tiles_w;
+  const int th = t % tiles_h;
+  t /= tiles_h;
+  const int d = t % D;
+  t /= D;
+  const int head = t % heads, b = t / heads;
+  const int h0 = th * 2 * BH, w0 = tw * 2 * BW, rh = kh / 2, rw = KW / 2;
+  const int hs0 = clampi(h0 - rh, 0, H - HR);
+  const int ws0 = periodic ? w0 - rw : clampi(w0 - rw, 0, W - WC);
+  const int ld0 = clampi(d - kd / 2, 0, D - kd);
+  const int nthr = blockDim.x >> 1;                       // threads of a half
+  const int half = threadIdx.x >= nthr ? 1 : 0, ht = threadIdx.x - half * nthr;
+  const int part = ht % TPB, blk = ht / TPB;
+  const int bh = h0 + 2 * (blk / BW), bw = w0 + 2 * (blk % BW);
+  const int own = 2 * (part & 1) + ((part >> 1) & 1);     // this thread's query: row own / 2, column own % 2
+  auto row_start = [&](int h) { return clampi(min(h, H - 1) - rh, 0, H - kh) - hs0; };
+  auto col_start = [&](int w) { return (periodic ? min(w, W - 1) - rw : clampi(min(w, W - 1) - rw, 0, W - KW)) - ws0; };
+  int ra = row_start(bh), cb = col_start(bw);             // the block's first key row and column
+  const int dr = row_start(bh + (own >> 1)) - ra, dc = col_start(bw + (own & 1)) - cb;
+  bool ok = true;
+  // debug builds: the block's windows lie in the slab
+  if (!WM_DCHECK(ra >= 0 && ra + dr + kh <= HR && cb >= 0 && cb + dc + KW <= WC && dr >= 0 && dr <= 1 && dc >= 0 &&
+                     dc <= 1 && ld0 >= 0 && ld0 + kd <= D,
+                 dstatus)) {
+    ra = cb = 0;
+    ok = false;
+  }
+  const uint32_t cmask = ((1u << KW) - 1u) << dc;
+  const long N = (long)D * H * W, C3 = 3L * C;
+  const float scale = rsqrtf((float)DH);
+  uint64_t q[4][2 * NI], o[4][2 * NI];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int qi = own ^ k, hq = min(bh + (qi >> 1), H - 1), wq = min(bw + (qi & 1), W - 1);
+    const ulonglong2* src = reinterpret_cast<const ulonglong2*>(qkv + ((long)b * N + ((long)d * H + hq) * W + wq) * C3 +
+                                                                head * DH);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const ulonglong2 v = src[i * TPB + part];
+      q[k][2 * i] = v.x;
+      q[k][2 * i + 1] = v.y;
+      o[k][2 * i] = o[k][2 * i + 1] = 0ull;
+    }
+  }
+  float m = -3.402823466e38f, l = 0.f;
+  const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(sm);
+  const int rows0 = (kh + 2) / 2;                         // rows of the first half; the second has kh + 1 - rows0
+  for (int li = 0; li < kd; ++li) {
+    __syncthreads();   // the previous level's slabs are no longer read
+    const long lev = (long)b * D + ld0 + li;
+    // a thread brings one 16-byte unit of a column of K or V, row after row
+    for (int idx = threadIdx.x; idx < 2 * WC * NU; idx += blockDim.x) {
+      const int c2 = idx / NU, u = idx - c2 * NU, kv = c2 >= WC ? 1 : 0, c = c2 - kv * WC;
+      int lon = ws0 + c;
+      while (lon < 0) lon += W;
+      while (lon >= W) lon -= W;
+      const float* src = qkv + ((lev * H + hs0) * W + lon) * C3 + (1 + kv) * C + head * DH + 4 * u;
+      uint32_t dst = smem0 + (uint32_t)(kv * vs + c * KS + 4 * u) * 4u;
+#pragma unroll 4
+      for (int r = 0; r < HR; ++r) {
+        cp_async16(dst, src);
+        src += (long)W * C3;
+        dst += (uint32_t)(WC * KS) * 4u;
+      }
+    }
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const int a_end = half ? kh + 1 : rows0;
+#pragma unroll 1
+    for (int a = half ? rows0 : 0; a < a_end; ++a) {
+      const uint32_t krow = smem0 + (uint32_t)((min(ra + a, HR - 1) * WC + cb) * KS + 4 * part) * 4u;
+      const uint32_t vrow = krow + (uint32_t)vs * 4u;
+      const uint32_t cm = a >= dr && a < dr + kh ? cmask : 0u;   // columns of this thread's query
+      float sc[NC], rmax = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        uint64_t s2[4];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          uint64_t k0, k1;
+          lds_f2(krow + (uint32_t)(j * KS + 4 * i * TPB) * 4u, k0, k1);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            s2[k] = i == 0 ? mul2(q[k][0], k0) : fma2(q[k][2 * i], k0, s2[k]);
+            s2[k] = fma2(q[k][2 * i + 1], k1, s2[k]);
+          }
+        }
+        float f[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 u = unpack2(s2[k]);
+          f[k] = u.x + u.y;
+        }
+        f[0] += __shfl_xor_sync(0xffffffffu, f[2], 1);
+        f[1] += __shfl_xor_sync(0xffffffffu, f[3], 1);
+        f[0] += __shfl_xor_sync(0xffffffffu, f[1], 2);
+        if constexpr (TPB == 8) f[0] += __shfl_xor_sync(0xffffffffu, f[0], 4);
+        sc[j] = (cm >> j) & 1u ? f[0] * scale : -INFINITY;
+        rmax = fmaxf(rmax, sc[j]);
+      }
+      // The reference moves only when some score of the warp passes it by more
+      // than 8 (probabilities stay below e^8), so most rows rescale nothing.
+      if (__any_sync(0xffffffffu, rmax > m + 8.f)) {
+        const float mn = fmaxf(m, rmax);
+        const float a0 = expf(m - mn);   // 0 while m is the initial value: o and l are still zero
+        l *= a0;
+        m = mn;
+        const float a1 = __shfl_xor_sync(0xffffffffu, a0, 2), a2 = __shfl_xor_sync(0xffffffffu, a0, 1),
+                    a3 = __shfl_xor_sync(0xffffffffu, a1, 1);
+        const uint64_t al[4] = {pack_f2(a0, a0), pack_f2(a1, a1), pack_f2(a2, a2), pack_f2(a3, a3)};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int i = 0; i < 2 * NI; ++i) o[k][i] = mul2(o[k][i], al[k]);
+      }
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const float p0 = expf(sc[j] - m);
+        l += p0;
+        const float p1 = __shfl_xor_sync(0xffffffffu, p0, 2), p2 = __shfl_xor_sync(0xffffffffu, p0, 1),
+                    p3 = __shfl_xor_sync(0xffffffffu, p1, 1);
+        const uint64_t pp[4] = {pack_f2(p0, p0), pack_f2(p1, p1), pack_f2(p2, p2), pack_f2(p3, p3)};
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          uint64_t v0, v1;
+          lds_f2(vrow + (uint32_t)(j * KS + 4 * i * TPB) * 4u, v0, v1);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            o[k][2 * i] = fma2(pp[k], v0, o[k][2 * i]);
+            o[k][2 * i + 1] = fma2(pp[k], v1, o[k][2 * i + 1]);
+          }
+        }
+      }
+    }
+  }
+  // the halves' softmax states, merged by the first half
+  __syncthreads();
+  float* xs = sm;
+  if (half) {
+    xs[ht] = m;
+    xs[nthr + ht] = l;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int i = 0; i < 2 * NI; ++i) {
+        const float2 u = unpack2(o[k][i]);
+        xs[(2 + 4 * NI * k + 2 * i) * nthr + ht] = u.x;
+        xs[(3 + 4 * NI * k + 2 * i) * nthr + ht] = u.y;
+      }
+  }
+  __syncthreads();
+  if (half) return;
+  const float m1 = xs[ht], M = fmaxf(m, m1);
+  const float e0 = expf(m - M), e1 = expf(m1 - M);
+  const float inv = 1.f / (l * e0 + xs[nthr + ht] * e1);
+  float f0[4], f1[4];   // weights of the two halves, divided by the sum
+  f0[0] = e0 * inv;
+  f1[0] = e1 * inv;
+  f0[1] = __shfl_xor_sync(0xffffffffu, f0[0], 2);
+  f1[1] = __shfl_xor_sync(0xffffffffu, f1[0], 2);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    f0[2 + k] = __shfl_xor_sync(0xffffffffu, f0[k], 1);
+    f1[2 + k] = __shfl_xor_sync(0xffffffffu, f1[k], 1);
+  }
+  uint32_t nan = 0u;   // float4 of a query at bit k NI + i
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int qi = own ^ k, hq = bh + (qi >> 1), wq = bw + (qi & 1);
+    if (!ok || hq >= H || wq >= W) continue;
+    float* orow = out + ((long)b * N + ((long)d * H + hq) * W + wq) * C + head * DH;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      float y[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 u = unpack2(o[k][2 * i + (e >> 1)]);
+        y[e] = ((e & 1) ? u.y : u.x) * f0[k] + xs[(2 + 4 * NI * k + 4 * i + e) * nthr + ht] * f1[k];
+        if (y[e] != y[e]) nan |= 1u << (k * NI + i);
+      }
+      *reinterpret_cast<float4*>(orow + 4 * (i * TPB + part)) = make_float4(y[0], y[1], y[2], y[3]);
+    }
+  }
+#pragma unroll 1
+  for (; nan != 0u; nan &= nan - 1u) {
+    const int bit = __ffs(nan) - 1, qi = own ^ (bit / NI), hq = bh + (qi >> 1), wq = bw + (qi & 1);
+    const long tok = (long)b * N + ((long)d * H + hq) * W + wq;
+    na_f32_query(qkv + tok * C3 + head * DH, qkv + (long)b * N * C3 + C + head * DH, out + tok * C + head * DH,
+                 4 * ((bit % NI) * TPB + part), H, W, C, DH, ld0, kd, row_start(bh + (qi >> 1)) + hs0, kh,
+                 col_start(bw + (qi & 1)) + ws0, KW, scale);
+  }
+}
+
+// Tile of the block kernel (blocks along latitude and longitude), its shared
+// memory and its CTAs; false if the shape is not its own.
+static bool na_f32_block_plan(int B, int D, int H, int W, int heads, int dh, int kh, int kw, bool periodic, int* BH,
+                              int* BW, size_t* smem, long* ctas) {
+  if ((kw != 3 && kw != 5 && kw != 7) || (dh != 16 && dh != 32 && dh != 48 && dh != 64)) return false;
+  const int wide = dh == 64 ? 4 : dh == 48 ? 6 : 8;
+  const int cand[3][2] = {{8, wide}, {4, wide}, {4, dh == 64 ? 2 : 4}};
+  const int tpb = dh == 64 ? 8 : 4, ks = dh == 64 ? 64 : dh + 8, maxt = dh == 48 ? 384 : 512;
+  double best = 0.0;
+  for (const auto& c : cand) {
+    const int HR = std::min(2 * c[0] + kh - 1, H), WC = periodic ? 2 * c[1] + kw - 1 : std::min(2 * c[1] + kw - 1, W);
+    const int threads = 2 * c[0] * c[1] * tpb;
+    const size_t bytes = std::max(((size_t)2 * HR * WC + 1) * ks * 4, (size_t)threads / 2 * (dh / tpb * 4 + 2) * 4);
+    if (bytes > 227 * 1024) continue;
+    const long n = (long)((H + 2 * c[0] - 1) / (2 * c[0])) * ((W + 2 * c[1] - 1) / (2 * c[1])) * D * heads * B;
+    const long per_sm = std::min<long>(maxt / threads, (227 * 1024) / (bytes + 1024));
+    const long waves = (n + num_sms() * per_sm - 1) / (num_sms() * per_sm);
+    // clocks of a CTA and level: its keys' FMAs, and its slab's way into shared
+    // memory (64 bytes a clock), which another CTA of the SM can hide
+    const double fma = (double)c[0] * c[1] * (kh + 1) * (kw + 1) * dh / 12.0, load = 2.0 * HR * WC * dh * 4 / 64;
+    // fewer than 12 warps on an SM leave issue slots empty
+    const double thin = std::max(1.0, 384.0 / (double)(per_sm * threads));
+    const double cost = (double)waves * (per_sm > 1 ? std::max(per_sm * fma * thin, per_sm * load) : fma * thin + load);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      *BH = c[0];
+      *BW = c[1];
+      *smem = bytes;
+      *ctas = n;
+    }
+  }
+  return best != 0.0;
+}
+
+template <int DH>
+static wm_status launch_na_f32_block(const float* qkv, float* out, int D, int H, int W, int C, int heads, int kd,
+                                     int kh, int kw, bool periodic, int BH, int BW, size_t smem, long ctas,
+                                     cudaStream_t s) {
+  const int tiles_h = (H + 2 * BH - 1) / (2 * BH), tiles_w = (W + 2 * BW - 1) / (2 * BW);
+  const dim3 grid((unsigned)ctas), block(2 * BH * BW * NaBlk<DH>::TPB);
+  auto kern = kw == 3 ? na_f32_block_kernel<DH, 3> : kw == 5 ? na_f32_block_kernel<DH, 5> : na_f32_block_kernel<DH, 7>;
+  kern<<<grid, block, smem, s>>>(qkv, out, D, H, W, C, heads, kd, kh, periodic ? 1 : 0, BH, BW, tiles_h, tiles_w,
+                                 device_status_word());
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
 // Shared memory of the tiled FP32 attention (K and V slabs), or 0 if the
 // shape does not fit it.
 static size_t na_f32_tile_smem(int H, int W, int dh, int kh, int kw, bool periodic) {
@@ -484,7 +821,20 @@ static size_t na_f32_tile_smem(int H, int W, int dh, int kh, int kw, bool period
   return bytes <= 227 * 1024 ? bytes : 0;
 }
 
+template <int DH>
+static wm_status prepare_na_f32_block() {
+  WM_CUDA(cudaFuncSetAttribute(na_f32_block_kernel<DH, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  WM_CUDA(cudaFuncSetAttribute(na_f32_block_kernel<DH, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  WM_CUDA(cudaFuncSetAttribute(na_f32_block_kernel<DH, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  return WM_OK;
+}
+
 wm_status prepare_na_f32() {
+  wm_status st = prepare_na_f32_block<16>();
+  if (st == WM_OK) st = prepare_na_f32_block<32>();
+  if (st == WM_OK) st = prepare_na_f32_block<48>();
+  if (st == WM_OK) st = prepare_na_f32_block<64>();
+  if (st != WM_OK) return st;
   WM_CUDA(cudaFuncSetAttribute(na_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   WM_CUDA(cudaFuncSetAttribute(na_f32_tile_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   WM_CUDA(cudaFuncSetAttribute(na_f32_tile_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
@@ -498,8 +848,21 @@ wm_status launch_na_f32(const float* qkv, float* out, int B, int D, int H, int W
   const long total = (long)B * D * H * W * heads;
   if (total <= 0) return WM_OK;
   const int dh0 = C / heads;
+  const bool aligned = C % 4 == 0 && ((uintptr_t)qkv & 15) == 0 && ((uintptr_t)out & 15) == 0;
+  int BH = 0, BW = 0;
+  size_t bsm = 0;
+  long bctas = 0;
+  if (aligned && na_f32_block_plan(B, D, H, W, heads, dh0, kh, kw, periodic, &BH, &BW, &bsm, &bctas)) {
+    if (bctas > (1L << 31) - 1) return fail(WM_ERR_INVALID_ARG, "too many attention tiles");
+    switch (dh0) {
+      case 16: return launch_na_f32_block<16>(qkv, out, D, H, W, C, heads, kd, kh, kw, periodic, BH, BW, bsm, bctas, s);
+      case 32: return launch_na_f32_block<32>(qkv, out, D, H, W, C, heads, kd, kh, kw, periodic, BH, BW, bsm, bctas, s);
+      case 48: return launch_na_f32_block<48>(qkv, out, D, H, W, C, heads, kd, kh, kw, periodic, BH, BW, bsm, bctas, s);
+      default: return launch_na_f32_block<64>(qkv, out, D, H, W, C, heads, kd, kh, kw, periodic, BH, BW, bsm, bctas, s);
+    }
+  }
   const size_t tsm = na_f32_tile_smem(H, W, dh0, kh, kw, periodic);
-  if (tsm && (C % 4) == 0 && (reinterpret_cast<uintptr_t>(qkv) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+  if (tsm && aligned) {
     const int tiles_h = (H + 7) / 8, tiles_w = (W + 7) / 8;
     const long ctas = (long)tiles_h * tiles_w * D * heads * B;
     if (ctas > (1L << 31) - 1) return fail(WM_ERR_INVALID_ARG, "too many attention tiles");
