@@ -649,9 +649,11 @@ wm_status block_forward(wm_ctx* ctx, float* x, int batch, int which, int b, bool
 int rollout_small_group(const wm_ctx* ctx, int batch);
 wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* n1, int G, cudaStream_t s);
 
-wm_status processor_step(wm_ctx* ctx, float* x, int batch, int which, cudaStream_t s) {
+// *per_kernel (may be NULL): whether the blocks ran kernel by kernel.
+wm_status processor_step(wm_ctx* ctx, float* x, int batch, int which, cudaStream_t s, bool* per_kernel = nullptr) {
   wm::NvtxRange range(which == WM_P6 ? "six-hour step" : "one-hour step");
   const int G = rollout_small_group(ctx, batch);
+  if (per_kernel) *per_kernel = G == 0;
   if (G > 0) {
     // narrow latent: the step's blocks as one whole-rollout launch per G latents
     const size_t lat = (size_t)ctx->N * ctx->cfg.C;
@@ -829,6 +831,17 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
 }  // namespace
 
 namespace wm {
+wm_status processor_step_copy(wm_ctx* ctx, float* x, int batch, int which, cudaStream_t s, const bf16** copy) {
+  *copy = nullptr;
+  WM_TRY(check_compute(ctx, x, batch));
+  std::lock_guard<std::recursive_mutex> lk(ctx->mu);
+  WM_TRY(ensure_workspace(ctx, batch));
+  bool per_kernel = false;
+  WM_TRY(processor_step(ctx, x, batch, which, s, &per_kernel));
+  if (per_kernel && ctx->cfg.precision != WM_PREC_FP32) *copy = ctx->xb;
+  return WM_OK;
+}
+
 bool processor_step_inplace_ok(wm_ctx* ctx, int n) {
   std::lock_guard<std::recursive_mutex> lk(ctx->mu);
   return n >= 1 && rollout_small_group(ctx, n) >= 1;

@@ -8,6 +8,7 @@
 // stack holds the encoder's blocks; the output map is one more GEMM. The
 // decoder runs the one-hour stack of the same wm_ctx and scatters the
 // transposed convolutions' outputs (one GEMM per part) back to the grid.
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -142,6 +143,168 @@ __global__ void unpatch_sfc_kernel(const float* __restrict__ y, float* __restric
 
 unsigned blocks_for(long total) { return (unsigned)((total + 255) / 256); }
 
+// The same four maps in units of U consecutive values of a field row (4 or 8
+// floats, one or two 128-bit loads), one grid row (blockIdx.y) per field row,
+// so that a thread divides by the patch width once for U values instead of
+// four to six times for one. A field row is a run of p v-wide pieces, one per
+// token, each contiguous in the patch matrix: U divides p v (atmosphere), or
+// the channels of each source (surface). Bound by HBM: fields of 28 x 720 x
+// 1440 x 5 into bf16 patches took 1.43 ms one value a thread (0.9 GB, 0.64
+// TB/s, all of it index arithmetic); the pieces' 80-byte rows meet in L2.
+// The whole 0.25-degree encode went from 10.0 to 8.6 ms, the decode from 9.75 to
+// 8.78 ms (with the residual copy of `blocks` below: 0.25 ms of each).
+template <int U, typename T>
+__device__ __forceinline__ void put(T* out, const float (&x)[U]) {
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int i = 0; i < U; i += 4) *reinterpret_cast<float4*>(out + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  } else {
+    uint32_t w[U / 2];
+#pragma unroll
+    for (int i = 0; i < U; i += 2) {
+      const __nv_bfloat162 b = __floats2bfloat162_rn(x[i], x[i + 1]);
+      w[i / 2] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    if constexpr (U == 8) *reinterpret_cast<uint4*>(out) = make_uint4(w[0], w[1], w[2], w[3]);
+    else *reinterpret_cast<uint2*>(out) = make_uint2(w[0], w[1]);
+  }
+}
+template <int U>
+__device__ __forceinline__ void take(float (&x)[U], const float* in) {
+#pragma unroll
+  for (int i = 0; i < U; i += 4) {
+    const float4 t = __ldcs(reinterpret_cast<const float4*>(in + i));
+    x[i] = t.x; x[i + 1] = t.y; x[i + 2] = t.z; x[i + 3] = t.w;
+  }
+}
+
+// rows: padded level x latitude of the grid; units: W0 v / U
+template <int U, typename T>
+__global__ void patch_atm_rows(const float* __restrict__ atm, T* __restrict__ out, int rows, int units, int H, int W,
+                               int H0, int pd, int p, int pv, int top) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= units) return;
+  const int w = u * U / pv, o = u * U - w * pv;   // token along the row, offset in its piece
+  const int K = pd * p * pv;
+  for (int row = blockIdx.y; row < rows; row += gridDim.y) {
+    const int lp = row / H0, y = row - lp * H0, h = y / p, l = lp / pd;
+    float x[U];
+    if (lp >= top) {
+      take(x, atm + ((long)(lp - top) * H0 + y) * (long)units * U + u * U);
+    } else {
+#pragma unroll
+      for (int i = 0; i < U; ++i) x[i] = 0.f;
+    }
+    put<U>(out + (((long)l * H + h) * W + w) * K + ((lp - l * pd) * p + (y - h * p)) * pv + o, x);
+  }
+}
+
+// rows: latitudes; units: W0 (vs + nc) / 4, of 4 channels of one pixel
+template <typename T>
+__global__ void patch_sfc_rows(const float* __restrict__ sfc, const float* __restrict__ cst, T* __restrict__ out,
+                               int rows, int units, int W, int W0, int p, int vs, int nc) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= units) return;
+  const int cin = vs + nc, x0 = u * 4 / cin, c = u * 4 - x0 * cin, w = x0 / p;
+  for (int y = blockIdx.y; y < rows; y += gridDim.y) {
+    const long pix = (long)y * W0 + x0;
+    float x[4];
+    take(x, c < vs ? sfc + pix * vs + c : cst + pix * nc + (c - vs));
+    const int h = y / p;
+    put<4>(out + ((long)h * W + w) * (p * p * cin) + ((y - h * p) * p + (x0 - w * p)) * cin + c, x);
+  }
+}
+
+// rows: output level x latitude; units: W0 v / U
+template <int U>
+__global__ void unpatch_atm_rows(const float* __restrict__ y, float* __restrict__ atm, int rows, int units, int H,
+                                 int W, int H0, int pd, int p, int pv, int top) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= units) return;
+  const int w = u * U / pv, o = u * U - w * pv;
+  for (int row = blockIdx.y; row < rows; row += gridDim.y) {
+    const int lev = row / H0, yy = row - lev * H0, lp = lev + top, l = lp / pd, h = yy / p;
+    float x[U];
+    take(x, y + (((long)l * H + h) * W + w) * (long)(pd * p * pv) + ((lp - l * pd) * p + (yy - h * p)) * pv + o);
+    put<U>(atm + (long)row * units * U + u * U, x);
+  }
+}
+
+bool aligned16(const void* a) { return (reinterpret_cast<uintptr_t>(a) & 15) == 0; }
+// Values per thread for rows of W0 v values in pieces of p v: 8, 4, or 0 where neither fits.
+int row_unit(int pv, const void* field, const void* patches) {
+  if (!aligned16(field) || !aligned16(patches)) return 0;
+  return pv % 8 == 0 ? 8 : pv % 4 == 0 ? 4 : 0;
+}
+dim3 row_grid(int units, int rows) {
+  return dim3((unsigned)((units + 127) / 128), (unsigned)std::min(rows, 32768));
+}
+
+template <typename T>
+wm_status patch_atm(const float* atm, T* out, const wm_codec_config& c, const Dims& d, cudaStream_t s) {
+  const int pv = c.p * c.v_atm, U = row_unit(pv, atm, out), top = c.level_pad - c.levels;
+  const long total = d.m_atm * d.k_atm;
+  if (total == 0) return WM_OK;
+  const int rows = c.level_pad * c.H0;
+  if (U == 8) {
+    const int units = c.W0 * c.v_atm / 8;
+    patch_atm_rows<8, T><<<row_grid(units, rows), 128, 0, s>>>(atm, out, rows, units, d.H, d.W, c.H0, c.pd, c.p, pv, top);
+  } else if (U == 4) {
+    const int units = c.W0 * c.v_atm / 4;
+    patch_atm_rows<4, T><<<row_grid(units, rows), 128, 0, s>>>(atm, out, rows, units, d.H, d.W, c.H0, c.pd, c.p, pv, top);
+  } else {
+    patch_atm_kernel<T><<<blocks_for(total), 256, 0, s>>>(atm, out, total, d.H, d.W, c.H0, c.W0, c.pd, c.p, c.v_atm, top);
+  }
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
+template <typename T>
+wm_status patch_sfc(const float* sfc, const float* cst, T* out, const wm_codec_config& c, const Dims& d,
+                    cudaStream_t s) {
+  const long total = d.m_sfc * d.k_sfc;
+  if (c.v_sfc_in % 4 == 0 && c.n_const % 4 == 0 && aligned16(sfc) && aligned16(cst) && aligned16(out)) {
+    const int units = c.W0 * (c.v_sfc_in + c.n_const) / 4;
+    patch_sfc_rows<T><<<row_grid(units, c.H0), 128, 0, s>>>(sfc, cst, out, c.H0, units, d.W, c.W0, c.p, c.v_sfc_in,
+                                                            c.n_const);
+  } else {
+    patch_sfc_kernel<T><<<blocks_for(total), 256, 0, s>>>(sfc, cst, out, total, d.W, c.W0, c.p, c.v_sfc_in, c.n_const);
+  }
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
+wm_status unpatch_atm(const float* y, float* atm, const wm_codec_config& c, const Dims& d, cudaStream_t s) {
+  const int pv = c.p * c.v_atm, U = row_unit(pv, atm, y), top = c.level_pad - c.levels, rows = c.levels * c.H0;
+  if (U == 8) {
+    const int units = c.W0 * c.v_atm / 8;
+    unpatch_atm_rows<8><<<row_grid(units, rows), 128, 0, s>>>(y, atm, rows, units, d.H, d.W, c.H0, c.pd, c.p, pv, top);
+  } else if (U == 4) {
+    const int units = c.W0 * c.v_atm / 4;
+    unpatch_atm_rows<4><<<row_grid(units, rows), 128, 0, s>>>(y, atm, rows, units, d.H, d.W, c.H0, c.pd, c.p, pv, top);
+  } else {
+    const long total = (long)c.levels * c.H0 * c.W0 * c.v_atm;
+    unpatch_atm_kernel<<<blocks_for(total), 256, 0, s>>>(y, atm, total, d.H, d.W, c.H0, c.W0, c.pd, c.p, c.v_atm, top);
+  }
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
+// The surface is the atmosphere of one level: latitude rows of W0 v values in pieces of p v.
+wm_status unpatch_sfc(const float* y, float* sfc, const wm_codec_config& c, const Dims& d, cudaStream_t s) {
+  const int pv = c.p * c.v_sfc_out, U = row_unit(pv, sfc, y);
+  if (U != 0) {
+    const int units = c.W0 * c.v_sfc_out / U;
+    auto kern = U == 8 ? unpatch_atm_rows<8> : unpatch_atm_rows<4>;
+    kern<<<row_grid(units, c.H0), 128, 0, s>>>(y, sfc, c.H0, units, d.H, d.W, c.H0, 1, c.p, pv, 0);
+  } else {
+    const long total = (long)c.H0 * c.W0 * c.v_sfc_out;
+    unpatch_sfc_kernel<<<blocks_for(total), 256, 0, s>>>(y, sfc, total, d.W, c.W0, c.p, c.v_sfc_out);
+  }
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
 }  // namespace
 
 struct wm_codec {
@@ -210,6 +373,20 @@ wm_status operand(const wm_codec* cd, const float* x, long n, const void** A, cu
   WM_TRY(wm::launch_f32_to_bf16(x, cd->xh, (size_t)n, s));
   *A = cd->xh;
   return WM_OK;
+}
+
+// The NA blocks of one stack on xe, and the GEMM operand of the result: the
+// bf16 copy that the last block's FC2 leaves beside its residual (the same
+// rounding of the same values as a pass over xe, 0.25 ms at 145,800 x 1024),
+// where the blocks ran kernel by kernel; else as `operand` makes it.
+wm_status blocks(const wm_codec* cd, int which, const void** A, cudaStream_t s) {
+  const bf16* copy = nullptr;
+  WM_TRY(wm::processor_step_copy(cd->inner, cd->xe, 1, which, s, &copy));
+  if (copy) {
+    *A = copy;
+    return WM_OK;
+  }
+  return operand(cd, cd->xe, cd->d.ntok * cd->cfg.Ce, A, s);
 }
 
 }  // namespace
@@ -296,27 +473,15 @@ wm_status wm_encode(wm_codec* cd, const float* atm, const float* sfc, const floa
   if ((c.v_sfc_in > 0 && !sfc) || (c.n_const > 0 && !consts)) return fail(WM_ERR_INVALID_ARG, "NULL surface input");
   cudaStream_t s = (cudaStream_t)stream;
   const bool bf = c.precision == WM_PREC_BF16;
-  const int top = c.level_pad - c.levels;
   // atmosphere: patch matrix, embedding GEMM into latent levels 0 .. D-2
-  long total = d.m_atm * d.k_atm;
-  if (bf) patch_atm_kernel<bf16><<<blocks_for(total), 256, 0, s>>>(atm, (bf16*)cd->patches, total, d.H, d.W, c.H0,
-                                                                    c.W0, c.pd, c.p, c.v_atm, top);
-  else patch_atm_kernel<float><<<blocks_for(total), 256, 0, s>>>(atm, (float*)cd->patches, total, d.H, d.W, c.H0,
-                                                                  c.W0, c.pd, c.p, c.v_atm, top);
-  WM_CUDA(cudaGetLastError());
+  WM_TRY(bf ? patch_atm(atm, (bf16*)cd->patches, c, d, s) : patch_atm(atm, (float*)cd->patches, c, d, s));
   WM_TRY(linear(cd, cd->patches, T_EMBED_ATM_W, T_EMBED_ATM_B, cd->xe, d.m_atm, c.Ce, d.k_atm, s));
   // surface + constants: the last latent level
-  total = d.m_sfc * d.k_sfc;
-  if (bf) patch_sfc_kernel<bf16><<<blocks_for(total), 256, 0, s>>>(sfc, consts, (bf16*)cd->patches, total, d.W,
-                                                                    c.W0, c.p, c.v_sfc_in, c.n_const);
-  else patch_sfc_kernel<float><<<blocks_for(total), 256, 0, s>>>(sfc, consts, (float*)cd->patches, total, d.W, c.W0,
-                                                                  c.p, c.v_sfc_in, c.n_const);
-  WM_CUDA(cudaGetLastError());
+  WM_TRY(bf ? patch_sfc(sfc, consts, (bf16*)cd->patches, c, d, s) : patch_sfc(sfc, consts, (float*)cd->patches, c, d, s));
   WM_TRY(linear(cd, cd->patches, T_EMBED_SFC_W, T_EMBED_SFC_B, cd->xe + d.m_atm * c.Ce, d.m_sfc, c.Ce, d.k_sfc, s));
   // NA blocks, then the map to the processor's width
-  WM_TRY(wm_processor_step(cd->inner, cd->xe, 1, WM_P6, stream));
   const void* A = nullptr;
-  WM_TRY(operand(cd, cd->xe, d.ntok * c.Ce, &A, s));
+  WM_TRY(blocks(cd, WM_P6, &A, s));
   return linear(cd, A, T_ENC_OUT_W, T_ENC_OUT_B, latent, d.ntok, c.C, c.Ce, s);
 }
 
@@ -328,23 +493,15 @@ wm_status wm_decode(wm_codec* cd, const float* latent, float* atm_out, float* sf
   const void* A = nullptr;
   WM_TRY(operand(cd, latent, d.ntok * c.C, &A, s));
   WM_TRY(linear(cd, A, T_DEC_IN_W, T_DEC_IN_B, cd->xe, d.ntok, c.Ce, c.C, s));
-  WM_TRY(wm_processor_step(cd->inner, cd->xe, 1, WM_P1, stream));
-  WM_TRY(operand(cd, cd->xe, d.ntok * c.Ce, &A, s));
+  WM_TRY(blocks(cd, WM_P1, &A, s));
   const size_t el = c.precision == WM_PREC_BF16 ? 2 : 4;
-  const int top = c.level_pad - c.levels;
   // atmosphere: one GEMM over levels 0 .. D-2, then the scatter to the grid
   WM_TRY(linear(cd, A, T_UNEMBED_ATM_W, T_UNEMBED_ATM_B, cd->outp, d.m_atm, d.k_atm, c.Ce, s));
-  long total = (long)c.levels * c.H0 * c.W0 * c.v_atm;
-  unpatch_atm_kernel<<<blocks_for(total), 256, 0, s>>>(cd->outp, atm_out, total, d.H, d.W, c.H0, c.W0, c.pd, c.p,
-                                                        c.v_atm, top);
-  WM_CUDA(cudaGetLastError());
+  WM_TRY(unpatch_atm(cd->outp, atm_out, c, d, s));
   // surface: the last latent level
   const void* As = (const char*)A + (size_t)d.m_atm * c.Ce * el;
   WM_TRY(linear(cd, As, T_UNEMBED_SFC_W, T_UNEMBED_SFC_B, cd->outp, d.m_sfc, d.n_sfc_out, c.Ce, s));
-  total = (long)c.H0 * c.W0 * c.v_sfc_out;
-  unpatch_sfc_kernel<<<blocks_for(total), 256, 0, s>>>(cd->outp, sfc_out, total, d.W, c.W0, c.p, c.v_sfc_out);
-  WM_CUDA(cudaGetLastError());
-  return WM_OK;
+  return unpatch_sfc(cd->outp, sfc_out, c, d, s);
 }
 
 wm_status wm_forecast_fields(wm_ctx* ctx, wm_codec* cd, const float* atm, const float* sfc, const float* consts,

@@ -82,8 +82,26 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ in, __nv_bfloat16* 
     out[i] = __float2bfloat16_rn(in[i]);
 }
 
+// Eight values a thread in 128-bit accesses: 145,800 x 768 in 190 us one value a thread.
+__global__ void f32_to_bf16_vec_kernel(const float4* __restrict__ in, uint4* __restrict__ out, size_t n8) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 a = __ldcs(in + 2 * i), b = __ldcs(in + 2 * i + 1);
+    const __nv_bfloat162 p0 = __floats2bfloat162_rn(a.x, a.y), p1 = __floats2bfloat162_rn(a.z, a.w);
+    const __nv_bfloat162 p2 = __floats2bfloat162_rn(b.x, b.y), p3 = __floats2bfloat162_rn(b.z, b.w);
+    out[i] = make_uint4(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1),
+                        *reinterpret_cast<const uint32_t*>(&p2), *reinterpret_cast<const uint32_t*>(&p3));
+  }
+}
+
 wm_status launch_f32_to_bf16(const float* in, __nv_bfloat16* out, size_t n, cudaStream_t s) {
   if (!n) return WM_OK;
+  if (n % 8 == 0 && (((uintptr_t)in | (uintptr_t)out) & 15) == 0) {
+    const int blocks = (int)std::min<size_t>((n / 8 + 255) / 256, (size_t)num_sms() * 32);
+    f32_to_bf16_vec_kernel<<<blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(in), reinterpret_cast<uint4*>(out),
+                                                  n / 8);
+    WM_CUDA(cudaGetLastError());
+    return WM_OK;
+  }
   const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)num_sms() * 8);
   f32_to_bf16_kernel<<<blocks, 256, 0, s>>>(in, out, n);
   WM_CUDA(cudaGetLastError());

@@ -20,6 +20,9 @@ const wm_config* ctx_config(const wm_ctx* ctx);
 // One processor step on `batch` contiguous latents, replayed from a CUDA graph
 // captured per (latent buffer, batch, processor, precision).
 wm_status processor_step_graphed(wm_ctx* ctx, float* x, int batch, int which, cudaStream_t s);
+// wm_processor_step; *copy: the bf16 copy of the result in the context's
+// workspace (until its next compute call), or NULL where the path makes none.
+wm_status processor_step_copy(wm_ctx* ctx, float* x, int batch, int which, cudaStream_t s, const __nv_bfloat16** copy);
 // The same for n latents at arbitrary device addresses, in place, when the
 // whole-rollout kernel takes the step (processor_step_inplace_ok).
 bool processor_step_inplace_ok(wm_ctx* ctx, int n);
