@@ -443,6 +443,15 @@ __global__ void __launch_bounds__(kThreads, 1) na_tc_kernel(const Params p) {
           }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
+        if (p.NS == 2) {
+          // Two stages: the next level waits for the level before this one to
+          // be consumed, and the MMAs that consume it are issued after one
+          // that needs this level, so this level cannot wait for the next.
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          fence_async_smem();
+          mbar_arrive(&kv_full[stage]);
+          continue;
+        }
         // the previous level's copies have landed: publish it to the MMA
         if (prev_stage >= 0) {
           asm volatile("cp.async.wait_group 1;" ::: "memory");
