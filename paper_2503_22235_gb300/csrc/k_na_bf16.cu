@@ -1054,30 +1054,92 @@ std::vector<NaPlan> na_candidates(int kh, int kw, int H, int W, int C, int heads
   return out;
 }
 
-// Heuristic when no tuned plan exists, among the plans of family `fam` (and
-// kernel kind `kind`, unless it is -1): fewest staged keys per query times
-// tile waste; persistent plans are preferred when the tile count gives every
-// SM several tiles.
-NaPlan na_heuristic(int B, int D, int H, int W, int heads, int kh, int kw, int dh, bool periodic, int fam, int kind) {
+// A plan's time in arbitrary units, for choosing one where none is tuned.
+// ceil(waves) times a CTA's work on its SM: a warp's MMAs of a tile (by
+// family), stretched as more than a few warps share a scheduler,
+// plus what the slabs' copies cost: little for a persistent CTA, whose ring
+// runs ahead, but much for its tiles that wrap in longitude (16-byte copies by
+// one warp), and in full for per-tile CTAs. The constants are fitted to the
+// tuner's times of every plan of 270 grids (2 x 16 x 32 x 128 to 9 x 90 x 180 x
+// 1024, windows 1 x 3 x 3 to 5 x 7 x 7, batches 1 to 4), for the picks' times.
+double na_plan_time(const NaPlan& pl, int B, int D, int H, int W, int heads, int kd, int kh, int kw, int dh,
+                    bool periodic) {
+  const int TH = pl.NWH * pl.WH, TW = pl.NWW * pl.WW, nw = pl.NWH * pl.NWW;
+  const int th = (H + TH - 1) / TH, tw = (W + TW - 1) / TW;
+  const int hr = std::min(TH + kh - 1, H), wc = (pl.NWW - 1) * pl.WW + pl.span;
+  const double ctas = (double)th * tw * D * B * heads;
+  const int regs = pl.gch == 8 && !pl.tr ? 168 : 128;
+  const long per_sm = pl.kind == 1 ? 1
+                                   : std::max<long>(1, std::min<long>(227 * 1024 / (long)(plan_smem(pl, kh, H, dh) + 1024),
+                                                                      65536 / (32 * nw * regs)));
+  const double on_sm = std::min((double)per_sm, std::ceil(ctas / num_sms()));
+  const double mma = (double)kd * ((std::min(pl.WH + kh - 1, H) * pl.span + 15) / 16) * (dh / 16) * (pl.tr ? 2 : 4);
+  const double per_mma = pl.tr ? (dh == 64 ? 0.426 : 0.778) : pl.gch == 8 ? (dh == 64 ? 0.526 : 0.842) : 1.0;
+  const double work = mma * per_mma + 27.6 * kd + (pl.tr ? 102.0 : 112.0);
+  const double lane = std::pow(std::pow(3.79, 1.69) + std::pow(nw * on_sm / 4.0, 1.69), 1.0 / 1.69);
+  const double load = (double)hr * wc * kd * dh;
+  double copies, start;
+  if (pl.kind == 1) {
+    int wraps = 0;
+    for (int t = 0; periodic && t < tw; ++t) wraps += t * TW - kw / 2 < 0 || t * TW - kw / 2 + wc > W;
+    copies = (0.00042 + 0.0715 * wraps / tw) * load;
+    start = 632.0;
+  } else {
+    copies = (on_sm > 1.0 ? 0.0229 * on_sm : 0.0272) * load;
+    start = 123.0;
+  }
+  const double waves = std::ceil(ctas / ((double)num_sms() * per_sm));
+  return (start + waves * (work * lane + copies)) * (pl.nbuf == 3 ? 0.963 : 1.0);
+}
+
+// Plan when none is tuned, among the plans of family `fam` (and kernel kind
+// `kind`, unless it is -1).
+NaPlan na_heuristic(int B, int D, int H, int W, int heads, int kd, int kh, int kw, int dh, bool periodic, int fam,
+                    int kind) {
   NaPlan best{};
-  double best_score = 1e30;
+  double best_t = 1e300;
   for (const NaPlan& pl : na_candidates(kh, kw, H, W, heads * dh, heads, periodic, fam)) {
     if (pl.tc) return pl;   // the tcgen05 family has one plan
     if (kind >= 0 && pl.kind != kind) continue;
-    const int TH = pl.NWH * pl.WH, TW = pl.NWW * pl.WW;
-    const int th = (H + TH - 1) / TH, tw = (W + TW - 1) / TW;
-    const int hr = std::min(TH + kh - 1, H), wc = (pl.NWW - 1) * pl.WW + pl.span;
-    const long ctas = (long)th * tw * D * B * heads;
-    double score = (double)hr * wc / (TH * TW) * ((double)th * TH / H) * ((double)tw * TW / W);
-    if (ctas < num_sms()) score *= (double)num_sms() / ctas;   // idle SMs
-    if (pl.kind == 1 && kind < 0) score *= (ctas >= 4L * num_sms()) ? 0.8 : 1.5;
-    score /= std::sqrt((double)(pl.NWH * pl.NWW * pl.WH * pl.WW) / 128.0);   // more warps hide more latency
-    if (score < best_score) {
-      best_score = score;
+    const double t = na_plan_time(pl, B, D, H, W, heads, kd, kh, kw, dh, periodic);
+    if (t < best_t) {
+      best_t = t;
       best = pl;
     }
   }
   return best;
+}
+
+// Arithmetic family of a shape that no context has tuned: the one of the plan
+// with the smallest time for one latent, so that a batched call rounds as a
+// single one does. With the plan chosen above, 1.04 times the fastest plan of
+// all on the 270 grids (1.27 with chunks of eight and the plan with the fewest
+// staged keys; 9 x 90 x 180 x 768: 1.58 ms, now 1.06), slower than those by
+// more than 2 % on six of them (at most 11 %).
+int na_default_family(int D, int H, int W, int heads, int kd, int kh, int kw, int dh, bool periodic) {
+  const NaPlan pl = na_heuristic(1, D, H, W, heads, kd, kh, kw, dh, periodic, 0, -1);
+  return pl.NWH ? family(pl) : 8;
+}
+
+// na_heuristic (fam = -1: of the default family), remembered per shape: the
+// candidates' times take ~10 us of host time, as long as a small launch.
+NaPlan na_pick(int B, int D, int H, int W, int C, int heads, int kd, int kh, int kw, bool periodic, int fam, int kind) {
+  static std::map<NaKey, NaPlan> picks;
+  constexpr size_t kMaxPicks = 4096;
+  NaKey key = na_key(B, D, H, W, C, heads, kd, kh, kw, periodic);
+  key[10] = 4 * (fam + 1) + kind + 1;
+  {
+    std::lock_guard<std::mutex> lk(g_na_mu);
+    auto it = picks.find(key);
+    if (it != picks.end()) return it->second;
+  }
+  const int dh = C / heads;
+  if (fam < 0) fam = na_default_family(D, H, W, heads, kd, kh, kw, dh, periodic);
+  const NaPlan pl = na_heuristic(B, D, H, W, heads, kd, kh, kw, dh, periodic, fam, kind);
+  std::lock_guard<std::mutex> lk(g_na_mu);
+  if (picks.size() >= kMaxPicks) picks.clear();
+  picks[key] = pl;
+  return pl;
 }
 
 template <int DH, int LS, int G, int MT, bool TR>
@@ -1193,9 +1255,9 @@ wm_status launch_na_bf16(const __nv_bfloat16* qkv, __nv_bfloat16* out, int B, in
     auto it = g_na_plans.find(na_key(B, D, H, W, C, heads, kd, kh, kw, periodic));
     if (it != g_na_plans.end()) pl = it->second;
     auto ig = g_na_family.find(na_key(0, D, H, W, C, heads, kd, kh, kw, periodic));
-    if (ig != g_na_family.end()) fam = ig->second;
+    fam = ig != g_na_family.end() ? ig->second : -1;
   }
-  if (!pl.NWH) pl = na_heuristic(B, D, H, W, heads, kh, kw, dh, periodic, fam, kind);
+  if (!pl.NWH) pl = na_pick(B, D, H, W, C, heads, kd, kh, kw, periodic, fam, kind);
   if (!pl.NWH) return fail(WM_ERR_INVALID_ARG, "attention window too large for the BF16 attention kernel");
   return launch_with(pl, make_params(qkv, out, B, D, H, W, C, heads, kd, kh, kw, periodic), dh, s, pdl);
 }
