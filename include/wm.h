@@ -373,7 +373,8 @@ wm_status wm_set_fused_mlp(int enable);
  * longitude, no rotary embedding, H % 8 == 0, W % 16 == 0, W >= 32 and
  * latitude / longitude windows of at most 5 as ONE kernel launch per group of
  * latents (as many as the device holds at once: 4 for the 4 x 24 x 48 latent).
- * Each CTA keeps an 8 x 16-token patch of its latent's residual stream in
+ * Each CTA keeps an 8 x 16-token patch (8 x 8 or 8 x 4 where few latents share
+ * the launch; same results) of its latent's residual stream in
  * shared memory for the whole rollout and runs every block's attention,
  * projection, MLP, LayerNorms and residual adds; the latent's CTAs meet once
  * per block at a counter in global memory. The result equals the per-kernel

@@ -97,6 +97,9 @@ struct wm_ctx {
   float* d_rs_qkv = nullptr;              // its double-buffered bf16 q, k, v (capacity in floats)
   size_t rs_qkv_cap = 0;
   unsigned int* d_rs_bar = nullptr;       // one barrier counter per latent
+  unsigned int* h_rs_done = nullptr;      // pinned: the last launch that has ended
+  unsigned int rs_seq = 0;                // the last launch made, and its stream (under g_rollout_traffic.mu)
+  cudaStream_t rs_stream = nullptr;
   std::recursive_mutex mu;
 };
 
@@ -713,7 +716,7 @@ wm_status run_graph(wm_ctx* ctx, const std::vector<uintptr_t>& key, cudaStream_t
 
 // ---- whole-rollout kernel for narrow latents
 
-// Patches of 8 x 16 tokens tile every level; the latitude halo of every patch
+// Patches of 8 x 16 tokens (hence the smaller ones) tile every level; the latitude halo of every patch
 // row spans 8 to 12 rows (a warp's 8-row key rectangle fits in it).
 bool rollout_small_shape(const wm_config& c) {
   if (c.precision != WM_PREC_BF16 || c.C != 128 || c.heads != 4 || !c.lon_periodic || c.rope) return false;
@@ -733,7 +736,7 @@ bool rollout_small_fits(const wm_ctx* ctx, int G) {
   if (g_fused_rollout.load() == 0 || ctx->timing || !rollout_small_shape(ctx->cfg)) return false;
   if (G < 1 || G > wm::kRolloutSmallMaxLatents) return false;
   const int T = ctx->cfg.D * (ctx->cfg.H / 8) * (ctx->cfg.W / 16);
-  return G * T <= wm::rollout_small_capacity();
+  return G * T <= wm::rollout_small_capacity(128);
 }
 
 // Latents per whole-rollout launch for `batch` latents of this context: the
@@ -742,8 +745,51 @@ bool rollout_small_fits(const wm_ctx* ctx, int G) {
 int rollout_small_group(const wm_ctx* ctx, int batch) {
   if (batch < 1 || !rollout_small_fits(ctx, 1)) return 0;
   const int T = ctx->cfg.D * (ctx->cfg.H / 8) * (ctx->cfg.W / 16);
-  return std::min({batch, wm::kRolloutSmallMaxLatents, wm::rollout_small_capacity() / T});
+  return std::min({batch, wm::kRolloutSmallMaxLatents, wm::rollout_small_capacity(128) / T});
 }
+
+// How many streams have whole-rollout launches in flight at once: the most
+// seen at any of the last eight launches.
+struct RolloutTraffic {
+  std::mutex mu;
+  std::vector<wm_ctx*> users;   // contexts that hold the kernel's weights
+  int recent[8] = {};
+  unsigned int n = 0;
+
+  void join(wm_ctx* ctx) {
+    std::lock_guard<std::mutex> lk(mu);
+    users.push_back(ctx);
+  }
+  void leave(wm_ctx* ctx) {
+    std::lock_guard<std::mutex> lk(mu);
+    users.erase(std::remove(users.begin(), users.end(), ctx), users.end());
+  }
+  // A launch of ctx on s is about to be made: its number, and the streams that share the device (s included).
+  int enter(wm_ctx* ctx, cudaStream_t s, unsigned int* seq) {
+    std::lock_guard<std::mutex> lk(mu);
+    std::vector<cudaStream_t> busy = {s};
+    for (const wm_ctx* u : users)
+      if (u != ctx && *static_cast<const volatile unsigned int*>(u->h_rs_done) != u->rs_seq &&
+          std::find(busy.begin(), busy.end(), u->rs_stream) == busy.end())
+        busy.push_back(u->rs_stream);
+    recent[n++ % 8] = (int)busy.size();
+    ctx->rs_stream = s;
+    *seq = ++ctx->rs_seq;
+    return peak();
+  }
+  int seen() {
+    std::lock_guard<std::mutex> lk(mu);
+    return peak();
+  }
+  // The launch was not made.
+  void undo(wm_ctx* ctx) {
+    std::lock_guard<std::mutex> lk(mu);
+    --ctx->rs_seq;
+  }
+
+ private:
+  int peak() const { return std::max(1, *std::max_element(recent, recent + 8)); }
+} g_rollout_traffic;
 
 // Once per context: every block's weights as 12 swizzled bf16 chunks and the
 // per-block table the kernel reads.
@@ -775,6 +821,9 @@ wm_status prepare_rollout_small(wm_ctx* ctx) {
   WM_CUDA(cudaMemcpy(ctx->d_rs_blk, tab.data(), tab.size() * sizeof(wm::RolloutBlock), cudaMemcpyHostToDevice));
   WM_CUDA(cudaMalloc(&ctx->d_rs_bar, wm::kRolloutSmallMaxLatents * sizeof(unsigned int)));
   WM_CUDA(cudaDeviceSynchronize());
+  WM_CUDA(cudaHostAlloc(&ctx->h_rs_done, sizeof(unsigned int), cudaHostAllocDefault));
+  *ctx->h_rs_done = 0;
+  g_rollout_traffic.join(ctx);
   return WM_OK;
 }
 
@@ -807,7 +856,24 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   a.L6 = c.blocks_p6;
   a.L1 = c.blocks_p1;
   a.G = G;
-  a.T = c.D * (c.H / 8) * (c.W / 16);
+  // Fewer tokens a CTA shorten every phase of a block, so a launch takes the
+  // smallest patches whose CTAs are all on the device at once, with as many
+  // launches beside it as other streams were lately seen to have in flight
+  // (launches that fill the chip would take turns). us per block of
+  // 4 x 24 x 48: one latent 33.3 with 128-token patches, 16.9 with 32; two
+  // 33.3, and 22.0 with 64. Four contexts on four streams, one 64-block
+  // rollout each: 2213 us with 128, 4288 with 32.
+  const bool counted = cap == cudaStreamCaptureStatusNone;   // a captured launch runs later, any number of times
+  const int streams = counted ? g_rollout_traffic.enter(ctx, s, &a.seq) : g_rollout_traffic.seen();
+  if (counted) a.done = ctx->h_rs_done;
+  struct Undo {
+    wm_ctx* ctx;
+    ~Undo() { if (ctx) g_rollout_traffic.undo(ctx); }
+  } undo{counted ? ctx : nullptr};
+  a.tokens = 128;
+  for (int t : {64, 32})
+    if (streams * G * c.D * (c.H / 8) * (c.W / (t / 8)) <= wm::rollout_small_capacity(t)) a.tokens = t;
+  a.T = c.D * (c.H / 8) * (c.W / (a.tokens / 8));
   a.D = c.D; a.H = c.H; a.W = c.W; a.kd = c.kd; a.kh = c.kh; a.kw = c.kw;
   for (int i = 0; i < G; ++i) {
     a.x[i] = x[i];
@@ -815,7 +881,7 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
     a.n1[i] = n1[i];
   }
   a.qkv = reinterpret_cast<bf16*>(ctx->d_rs_qkv);
-  const uint32_t box_w[3] = {20, 18, 2};
+  const uint32_t tw = (uint32_t)a.tokens / 8, box_w[3] = {tw + 4, tw + 2, 2};
   for (int k = 0; k < 3; ++k)
     if (!wm::make_tmap_kv_slab(&a.tm_kv[k], a.qkv, 384, (uint64_t)c.W, (uint64_t)c.H, 2ull * G * c.D, box_w[k], 12))
       return fail(WM_ERR_CUDA, "cuTensorMapEncodeTiled failed for the whole-rollout K/V rows");
@@ -825,7 +891,9 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   a.scale_log2 = (float)(1.4426950408889634 / std::sqrt(32.0));
   WM_CUDA(cudaMemsetAsync(ctx->d_rs_bar, 0, G * sizeof(unsigned int), s));
   wm::NvtxRange range("whole rollout (narrow latent)");
-  return wm::launch_rollout_small(a, s);
+  WM_TRY(wm::launch_rollout_small(a, s));
+  undo.ctx = nullptr;
+  return WM_OK;
 }
 
 }  // namespace
@@ -1161,6 +1229,8 @@ wm_status wm_destroy(wm_ctx* ctx) {
   cudaFree(ctx->d_rs_blk);
   cudaFree(ctx->d_rs_qkv);
   cudaFree(ctx->d_rs_bar);
+  g_rollout_traffic.leave(ctx);
+  cudaFreeHost(ctx->h_rs_done);
   cudaFree(ctx->d_stage);
   cudaFree(ctx->d_io);
   for (float* p : ctx->d_ring) cudaFree(p);

@@ -4,17 +4,19 @@
 // Why: at C = 128 a block's five GEMM / attention launches are each a few
 // microseconds of latency on a few dozen SMs, so a 14-day rollout (448 blocks)
 // is bound by launch and memory round trips, not by arithmetic. Here each CTA
-// owns one 8 x 16 (latitude x longitude) patch of 128 tokens of one level of
-// one latent for the whole rollout; its residual rows stay in tensor memory,
-// and per block (pre-LN transformer block, paper Sec. 2.1 and App. A.2):
+// owns one patch of 8 latitudes x 16, 8 or 4 longitudes (128, 64 or 32 tokens)
+// of one level of one latent for the whole rollout; its residual rows stay in
+// tensor memory, and per block (pre-LN transformer block, paper Sec. 2.1 and
+// App. A.2):
 //
 //   attention   8 warps, mma.sync m16n8k16: each warp takes a 4 x 4 query
-//               group and one head at a time and walks its 8 x 8 key
+//               group and one head at a time (64- and 32-token patches: two
+//               and four heads side by side) and walks its 8 x 8 key
 //               rectangle per key level (K/V slabs of the patch's halo brought
 //               to shared memory by tensor copies from a producer warp, one
-//               box per slab and two where the longitude wraps, three
-//               stages), FP32 online softmax; O goes to shared memory as the
-//               next GEMM's A operand
+//               box per slab and two where the longitude wraps, three or
+//               two stages), FP32 online softmax; O goes to shared memory as
+//               the next GEMM's A operand
 //   proj        tcgen05.mma (M = N = 128, K = 128) into TMEM; x += acc + b_o;
 //               LayerNorm 2 of the new rows (two-pass, FP32) -> bf16 A operand
 //   MLP         four 128-column hidden chunks: FC1 into two TMEM buffers,
@@ -30,14 +32,24 @@
 // block's weights (12 pre-swizzled 32 KB chunks per block, one bulk copy each,
 // through a two-slot ring) and its biases and LayerNorm vectors (one bulk
 // copy into a two-slot buffer), warp 10 one thread issuing the K/V tensor
-// copies into a three-stage ring. Latents are independent: each has its own
+// copies into the ring. Latents are independent: each has its own
 // schedule (six-hour blocks, then one-hour blocks) and its own barrier, so
 // latents with different lead times share the launch.
+//
+// A block's phases are chains of dependent latencies (attention 44 %, GELU
+// 21 %, QKV store 13 % of a 128-token patch's 67 k cycles; issue slots 41 %
+// busy), and one 4 x 24 x 48 latent in 128-token patches is 36 CTAs of 152
+// SMs: smaller patches put the idle SMs to work and shorten every phase but
+// the MMAs and the barrier. us per block: one latent 33.3 -> 16.9 (32 tokens,
+// 144 CTAs), two 33.3 -> 22.0 (64 tokens), three or four 33.6 as before (128 tokens).
+// All patch sizes round alike, so the results do not depend on the choice.
 //
 // Every mbarrier wait and the latent barrier are bounded in time; on a
 // timeout the CTA records WM_ERR_TIMEOUT, the compute warps leave together
 // (barrier with OR-reduction), copies and MMAs in flight are drained, TMEM
 // is freed and the CTA returns.
+#include <atomic>
+
 #include "tc_gemm.cuh"
 
 namespace wm {
@@ -49,30 +61,44 @@ using bf16 = __nv_bfloat16;
 using Blk = RolloutBlock;
 
 constexpr int C = 128, DH = 32, QKV = 3 * C;
-constexpr int TH = 8, TW = 16;                 // query patch of one CTA
-constexpr int SW = TW + 4;                     // slab columns: the patch's longitudes + 2 on each side
+constexpr int TH = 8;                          // latitudes of a patch
 constexpr int SR_MAX = TH + 4;                 // slab rows (latitude windows of at most 5)
 constexpr int THREADS = 352, MMA_WARP = 8, LOAD_WARP = 9, KV_WARP = 10;
 constexpr int CHUNK = 128 * 128 * 2;           // 128 x 128 bf16 operand: two 64-column 128B-swizzled slices
 constexpr int SLICE = CHUNK / 2;
 constexpr int NSLOT = 2;                       // weight ring slots
-constexpr int NKV = 3;                         // K/V stages
 constexpr int VEC_FLOATS = 1664;               // a block's vectors (layout below)
 constexpr int VEC_BYTES = VEC_FLOATS * 4;
 constexpr int OFF_A = 0;                       // A operand: LN1(x), O or LN2(x)
 constexpr int OFF_W = OFF_A + CHUNK;           // weight ring
-constexpr int OFF_H = OFF_W + NSLOT * CHUNK;   // GELU chunks, 2 slots; K/V stages 0 and 1 alias it
-constexpr int KV_SLAB = SR_MAX * SW * DH * 2;  // one head's K (or V) rows of a key level
-constexpr int KV_STAGE = 2 * KV_SLAB;
-constexpr int OFF_KV2 = OFF_H + 2 * CHUNK;     // the third K/V stage (the first two alias the GELU region)
-constexpr int OFF_VEC = OFF_KV2 + KV_STAGE;    // vectors of two blocks
-constexpr int SMEM_USED = OFF_VEC + 2 * VEC_BYTES;
-constexpr int SMEM = SMEM_USED + 1024;         // + alignment slack
-constexpr int OFF_RED = OFF_H + 2 * KV_STAGE;  // LayerNorm row partials [2 passes][2 halves][128]
-static_assert(OFF_RED + 4 * 128 * 4 <= OFF_H + 2 * CHUNK, "LayerNorm exchange must fit in the GELU region");
-static_assert(OFF_H % 1024 == 0 && OFF_KV2 % 512 == 0 && KV_SLAB % 512 == 0, "swizzled operands need aligned bases");
-static_assert(SMEM <= 232448, "shared memory per CTA");
-__device__ __forceinline__ uint32_t kv_stage_off(int b) { return (uint32_t)(b < 2 ? OFF_H + b * KV_STAGE : OFF_KV2); }
+constexpr int OFF_H = OFF_W + NSLOT * CHUNK;   // GELU chunks, 2 slots; the first K/V stages alias it
+
+// A patch of TP tokens: 8 latitudes x TP / 8 longitudes. The MMAs have 128
+// rows whatever TP is: NCP = 128 / TP copies of the patch's rows, and each
+// copy's threads take 1 / NCP of the columns of everything that is done per
+// element (bias, GELU, LayerNorm, residual); in attention the NCP head groups
+// of a step go to different warps.
+template <int TP>
+struct Cfg {
+  static constexpr int TW = TP / TH, SW = TW + 4;   // longitudes of the patch, of its slab (2 on each side)
+  static constexpr int NCP = 128 / TP, NC = 64 / NCP;   // copies; columns per epilogue thread
+  static constexpr int NH = 4 / NCP;                // heads a warp takes in turn
+  static constexpr int KV_SLAB = SR_MAX * SW * DH * 2;  // one head's K (or V) rows of a key level
+  static constexpr int KV_STAGE = 2 * NCP * KV_SLAB;    // K and V of the NCP heads of a step
+  static constexpr int NKV = TP == 128 ? 3 : 2;         // stages; NIN of them alias the GELU region
+  static constexpr int NIN = TP == 128 ? 2 : 1;
+  static constexpr int OFF_KV = OFF_H + 2 * CHUNK;      // the others
+  static constexpr int OFF_VEC = OFF_KV + (NKV - NIN) * KV_STAGE;   // vectors of two blocks
+  static constexpr int SMEM = OFF_VEC + 2 * VEC_BYTES + 1024;       // + alignment slack
+  static constexpr int OFF_RED = OFF_H + NIN * KV_STAGE;  // LayerNorm row partials [2 passes][2 halves][TP]
+  static_assert(OFF_RED + 4 * TP * 4 <= OFF_H + 2 * CHUNK, "LayerNorm exchange must fit in the GELU region");
+  static_assert(OFF_H % 1024 == 0 && OFF_KV % 512 == 0 && KV_SLAB % 512 == 0 && KV_STAGE % 512 == 0,
+                "swizzled operands need aligned bases");
+  static_assert(SMEM <= 232448, "shared memory per CTA");
+  static __device__ __forceinline__ uint32_t kv_stage_off(int b) {
+    return (uint32_t)(b < NIN ? OFF_H + b * KV_STAGE : OFF_KV + (b - NIN) * KV_STAGE);
+  }
+};
 // TMEM columns: FC1 accumulators (and the projection's) at 0 and 128, FC2's at
 // 256; QKV chunks at 0, 128, 256; the fp32 residual rows at 384
 constexpr uint32_t T_ACC1 = 0, T_PROJ = 0, T_ACC2 = 256, T_X = 384;
@@ -139,16 +165,45 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
-// 32 consecutive TMEM columns of this warp's 32 lanes (one row per thread); the caller waits (tmem_wait_st)
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
-      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "f"(v[16]), "f"(v[17]), "f"(v[18]),
-      "f"(v[19]), "f"(v[20]), "f"(v[21]), "f"(v[22]), "f"(v[23]), "f"(v[24]), "f"(v[25]), "f"(v[26]), "f"(v[27]),
-      "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31])
-      : "memory");
+// N = 16 or 32 consecutive TMEM columns of this warp's 32 lanes (one row per thread).
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]) {
+  if constexpr (N == 32) {
+    tmem_ld32(taddr, v);
+  } else {
+    static_assert(N == 16, "16 or 32 columns");
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  }
+}
+// The same to TMEM; the caller waits (tmem_wait_st).
+template <int N>
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[N]) {
+  if constexpr (N == 32) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "f"(v[16]), "f"(v[17]), "f"(v[18]),
+        "f"(v[19]), "f"(v[20]), "f"(v[21]), "f"(v[22]), "f"(v[23]), "f"(v[24]), "f"(v[25]), "f"(v[26]), "f"(v[27]),
+        "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31])
+        : "memory");
+  } else {
+    static_assert(N == 16, "16 or 32 columns");
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+        : "memory");
+  }
 }
 
 // byte offset of bf16 element (r, c) of a 128 x 128 operand (two 128B-swizzled 64-column slices)
@@ -162,63 +217,88 @@ __device__ __forceinline__ const bf16* block_weights(const RolloutSmallArgs& a, 
   return (i < p6 ? a.blk[i % a.L6] : a.blk[a.L6 + (i - p6) % a.L1]).w;
 }
 
-// LayerNorm of the thread's 64 columns (half hf of row r) with the partner
-// half's partial sums exchanged through shared memory (two passes: mean, then
-// the mean squared deviation), affine (gamma, beta: shared-memory vectors),
-// rounded to bf16 into the A operand.
-__device__ __forceinline__ void layernorm_to_a(uint8_t* smem, const float (&v)[64], int r, int hf,
+// The place of an epilogue thread: token tr of the patch (row copy * TP + tr of
+// the MMAs) and its columns c0 .. c0 + NC - 1, all in half hf of the 128.
+struct Place {
+  int tr, copy, hf, c0;
+};
+
+// LayerNorm of the thread's columns (two passes: mean, then the mean squared
+// deviation). A row's sum is the sum of its halves, each a chain of 64
+// additions in column order, whatever TP is, so that every patch size rounds
+// alike: a half's threads continue the chain one copy after the other through
+// shared memory. Affine (gamma, beta: shared-memory vectors), rounded to bf16
+// into the token's NCP rows of the A operand.
+template <int TP>
+__device__ __forceinline__ void layernorm_to_a(uint8_t* smem, const float (&v)[Cfg<TP>::NC], const Place& pl,
                                                const float4* gamma, const float4* beta, float eps) {
-  float* red = reinterpret_cast<float*>(smem + OFF_RED);
-  float s = 0.f;
+  using CF = Cfg<TP>;
+  constexpr int NC = CF::NC, NCP = CF::NCP;
+  float* red = reinterpret_cast<float*>(smem + CF::OFF_RED);
 #pragma unroll
-  for (int j = 0; j < 64; ++j) s += v[j];
-  red[hf * 128 + r] = s;
-  bar_compute();
-  const float mean = (red[r] + red[128 + r]) * (1.f / C);
-  float q = 0.f;
+  for (int c = 0; c < NCP; ++c) {
+    if (NCP == 1 || pl.copy == c) {
+      float s = c == 0 ? 0.f : red[pl.hf * TP + pl.tr];
 #pragma unroll
-  for (int j = 0; j < 64; ++j) {
-    const float dv = v[j] - mean;
-    q += dv * dv;
+      for (int j = 0; j < NC; ++j) s += v[j];
+      red[pl.hf * TP + pl.tr] = s;
+    }
+    bar_compute();
   }
-  red[256 + hf * 128 + r] = q;
-  bar_compute();
-  const float rstd = rsqrtf((red[256 + r] + red[384 + r]) * (1.f / C) + eps);
-  uint8_t* A = smem + OFF_A;
+  const float mean = (red[pl.tr] + red[TP + pl.tr]) * (1.f / C);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int j = 8 * k, c4 = (64 * hf + j) >> 2;
+  for (int c = 0; c < NCP; ++c) {
+    if (NCP == 1 || pl.copy == c) {
+      float q = c == 0 ? 0.f : red[(2 + pl.hf) * TP + pl.tr];
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const float dv = v[j] - mean;
+        q += dv * dv;
+      }
+      red[(2 + pl.hf) * TP + pl.tr] = q;
+    }
+    bar_compute();
+  }
+  const float rstd = rsqrtf((red[2 * TP + pl.tr] + red[3 * TP + pl.tr]) * (1.f / C) + eps);
+  uint8_t* A = smem + OFF_A + pl.hf * SLICE + pl.tr * 128;
+#pragma unroll
+  for (int k = 0; k < NC / 8; ++k) {
+    const int j = 8 * k, c4 = (pl.c0 + j) >> 2, u = (NC * pl.copy >> 3) + k;
     const float4 g0 = gamma[c4], g1 = gamma[c4 + 1];
     const float4 b0 = beta[c4], b1 = beta[c4 + 1];
     const uint32_t w0 = pack_bf16((v[j] - mean) * rstd * g0.x + b0.x, (v[j + 1] - mean) * rstd * g0.y + b0.y);
     const uint32_t w1 = pack_bf16((v[j + 2] - mean) * rstd * g0.z + b0.z, (v[j + 3] - mean) * rstd * g0.w + b0.w);
     const uint32_t w2 = pack_bf16((v[j + 4] - mean) * rstd * g1.x + b1.x, (v[j + 5] - mean) * rstd * g1.y + b1.y);
     const uint32_t w3 = pack_bf16((v[j + 6] - mean) * rstd * g1.z + b1.z, (v[j + 7] - mean) * rstd * g1.w + b1.w);
-    *reinterpret_cast<uint4*>(A + hf * SLICE + r * 128 + ((k ^ (r & 7)) << 4)) = make_uint4(w0, w1, w2, w3);
+#pragma unroll
+    for (int c = 0; c < NCP; ++c)
+      *reinterpret_cast<uint4*>(A + c * TP * 128 + ((u ^ (pl.tr & 7)) << 4)) = make_uint4(w0, w1, w2, w3);
   }
 }
 
-// x += acc + bias over the thread's 64 columns (TMEM accumulator at acc_col,
+// x += acc + bias over the thread's columns (TMEM accumulator at acc_col,
 // residual rows at T_X); the new values also into v.
-__device__ __forceinline__ void residual_add(uint32_t tmem, uint32_t lane_off, uint32_t acc_col, int hf,
-                                             const float4* bias, float (&v)[64]) {
+template <int TP>
+__device__ __forceinline__ void residual_add(uint32_t tmem, uint32_t lane_off, uint32_t acc_col, const Place& pl,
+                                             const float4* bias, float (&v)[Cfg<TP>::NC]) {
+  constexpr int NC = Cfg<TP>::NC, NS = NC < 32 ? NC : 32;
 #pragma unroll
-  for (int sub = 0; sub < 2; ++sub) {
-    const uint32_t col = (uint32_t)(64 * hf + 32 * sub);
-    float acc[32], x[32];
-    tmem_ld32(tmem + acc_col + col + lane_off, acc);
-    tmem_ld32(tmem + T_X + col + lane_off, x);
+  for (int sub = 0; sub < NC; sub += NS) {
+    const uint32_t col = (uint32_t)(pl.c0 + sub);
+    float acc[NS], x[NS];
+    tmem_ld<NS>(tmem + acc_col + col + lane_off, acc);
+    tmem_ld<NS>(tmem + T_X + col + lane_off, x);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < NS / 4; ++q) {
       const float4 b = bias[(col >> 2) + q];
       x[4 * q] += acc[4 * q] + b.x;
       x[4 * q + 1] += acc[4 * q + 1] + b.y;
       x[4 * q + 2] += acc[4 * q + 2] + b.z;
       x[4 * q + 3] += acc[4 * q + 3] + b.w;
     }
-    tmem_st32(tmem + T_X + col + lane_off, x);
+    tmem_st<NS>(tmem + T_X + col + lane_off, x);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[32 * sub + j] = x[j];
+    for (int j = 0; j < NS; ++j) v[sub + j] = x[j];
   }
   tmem_wait_st();
 }
@@ -255,7 +335,11 @@ __device__ __forceinline__ bool latent_barrier(unsigned int* counter, unsigned i
   return !bar_compute_or(!ok);
 }
 
+template <int TP>
 __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_constant__ RolloutSmallArgs a) {
+  using CF = Cfg<TP>;
+  constexpr int TW = CF::TW, SW = CF::SW, NC = CF::NC, NCP = CF::NCP, NH = CF::NH, NKV = CF::NKV;
+  constexpr int KV_SLAB = CF::KV_SLAB, OFF_VEC = CF::OFF_VEC, NS = NC < 32 ? NC : 32;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t w_full[NSLOT], w_empty[NSLOT], vec_full[2], vec_empty[2];
   __shared__ __align__(8) uint64_t a_full, mma_done, drain_bar, qkv_ready;
@@ -268,9 +352,9 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.x / a.T, tile = blockIdx.x % a.T;
   const int nb = a.n6[g] * a.L6 + a.n1[g] * a.L1;   // blocks of this latent's rollout (>= 1)
-  const int steps = 4 * a.kd;                         // attention steps per block: (head, key level)
+  const int steps = NH * a.kd;                        // attention steps per block: (head of each group, key level)
 
-  // the patch: level d, latitudes h0 .. h0 + 7, longitudes w0 .. w0 + 15; its
+  // the patch: level d, latitudes h0 .. h0 + 7, longitudes w0 .. w0 + TW - 1; its
   // key levels kd0 .. kd0 + kd - 1 and slab latitudes S0 .. S0 + SR - 1
   const int tpr = a.W / TW, tpl = (a.H / TH) * tpr;
   const int d = tile / tpl, h0 = ((tile % tpl) / tpr) * TH, w0 = (tile % tpr) * TW;
@@ -278,9 +362,9 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
   const int S0 = clampi(h0 - rh, 0, a.H - a.kh);
   const int SR = clampi(h0 + TH - 1 - rh, 0, a.H - a.kh) + a.kh - S0;
   const int kd0 = clampi(d - a.kd / 2, 0, a.D - a.kd);
-  // K/V slab layout: 12 latitude rows x 20 longitudes of 64-byte key rows, one
-  // box; where the patch's longitude halo wraps (w0 = 0 or W - 16), two boxes
-  // side by side: columns 0-1 then 2-19, or 0-17 then 18-19
+  // K/V slab layout: 12 latitude rows x SW longitudes of 64-byte key rows, one
+  // box; where the patch's longitude halo wraps (w0 = 0 or W - TW), two boxes
+  // side by side: two columns then the others, or the last two last
   const int wrap = w0 == 0 ? -1 : (w0 + TW + 2 > a.W ? 1 : 0);
 
   if (threadIdx.x == 0) {
@@ -374,8 +458,8 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       // ------------------------------------------------- K/V tensor copies
       for (int k = 0; k < 3; ++k) asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&a.tm_kv[k]) : "memory");
       // boxes of 12 latitudes from S0 (rows past H read as zeros, rows past SR
-      // are not used) x 20 longitudes, K and V
-      const uint32_t kv_bytes = (uint32_t)(SR_MAX * SW * 64 * 2);
+      // are not used) x SW longitudes, K and V of one head of each group
+      const uint32_t kv_bytes = (uint32_t)CF::KV_STAGE;
       int kst = 0, kpar = 0, last[NKV];   // ring position and its use parity
       for (int b = 0; b < NKV; ++b) last[b] = -1;
       bool ok = true;
@@ -395,18 +479,18 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
             ok = false;
             break;
           }
-          const int h = s / a.kd, lev = ((i & 1) * a.G + g) * a.D + kd0 + s % a.kd;
+          const int hi = s / a.kd, lev = ((i & 1) * a.G + g) * a.D + kd0 + s % a.kd;
           // debug builds: the boxes start inside the q, k, v array (a failed
           // check still issues the copies from coordinate 0, so the stage completes)
           const bool coords = WM_DCHECK(S0 >= 0 && S0 < a.H && lev >= 0 && lev < 2 * a.G * a.D &&
                                             (wrap != 0 || (w0 - 2 >= 0 && w0 - 2 + SW <= a.W)),
                                         a.status);
           mbar_expect_tx(&kv_full[b], kv_bytes);
-          const uint32_t dst0 = sbase + kv_stage_off(b);
+          const uint32_t dst0 = sbase + CF::kv_stage_off(b);
 #pragma unroll
-          for (int kv = 0; kv < 2; ++kv) {
-            const int ch = C + kv * C + h * DH;
-            const uint32_t dst = dst0 + kv * KV_SLAB;
+          for (int kk = 0; kk < 2 * NCP; ++kk) {   // K, V of head hi of group kk / 2
+            const int ch = C + (kk & 1) * C + ((kk >> 1) * NH + hi) * DH;
+            const uint32_t dst = dst0 + kk * KV_SLAB;
             if (!coords) {
               tma_load_4d(dst, &a.tm_kv[0], &kv_full[b], ch, 0, 0, 0);
             } else if (wrap == 0) {
@@ -415,8 +499,8 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
               tma_load_4d(dst, &a.tm_kv[2], &kv_full[b], ch, a.W - 2, S0, lev);
               tma_load_4d(dst + SR_MAX * 2 * 64, &a.tm_kv[1], &kv_full[b], ch, 0, S0, lev);
             } else {
-              tma_load_4d(dst, &a.tm_kv[1], &kv_full[b], ch, a.W - 18, S0, lev);
-              tma_load_4d(dst + SR_MAX * 18 * 64, &a.tm_kv[2], &kv_full[b], ch, 0, S0, lev);
+              tma_load_4d(dst, &a.tm_kv[1], &kv_full[b], ch, a.W - (SW - 2), S0, lev);
+              tma_load_4d(dst + SR_MAX * (SW - 2) * 64, &a.tm_kv[2], &kv_full[b], ch, 0, S0, lev);
             }
           }
           last[b] = (int)use;
@@ -510,17 +594,21 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
     }
   } else if (warp < 8) {
     // ------------------------------------------------------ compute warps
-    const int r = 32 * (warp & 3) + lane, hf = warp >> 2;   // epilogue row and column half
+    const int mr = 32 * (warp & 3) + lane;   // this thread's row of the MMAs
+    const int copy = NCP == 1 ? 0 : mr / TP, hf = warp >> 2;
+    const Place pl{NCP == 1 ? mr : mr % TP, copy, hf, 64 * hf + NC * copy};
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     const long N = (long)a.D * a.H * a.W;
-    const int tok_r = (d * a.H + h0 + (r >> 4)) * a.W + w0 + (r & 15);
-    float* xg = a.x[g] + (long)tok_r * C + 64 * hf;
+    const int tok_r = (d * a.H + h0 + pl.tr / TW) * a.W + w0 + pl.tr % TW;
+    float* xg = a.x[g] + (long)tok_r * C + pl.c0;
     int md = 0;          // mma_done completions waited for
     bool ok = true;
-    float v[64];
+    float v[NC];
 
     // attention geometry of this warp: a 4 x 4 query group (rows g8, g8 + 8 of the m16 tile)
-    const int gr = warp >> 2, gc = warp & 3, g8 = lane >> 2, t4 = lane & 3;
+    // of the patch's 2 x TW / 4, and one of the NCP head groups
+    const int grp = NCP == 1 ? warp : warp % (TP / 16), hs = NCP == 1 ? 0 : warp / (TP / 16);
+    const int gr = grp / (TW / 4), gc = grp % (TW / 4), g8 = lane >> 2, t4 = lane & 3;
     const int rw = a.kw / 2;
     int R0 = min(clampi(h0 + 4 * gr - rh, 0, a.H - a.kh) - S0, SR - 8);
     const int qh0 = h0 + 4 * gr + (g8 >> 2), qh1 = qh0 + 2, qcl = g8 & 3;
@@ -544,8 +632,8 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
     auto kv_off = [&](int lr, int c, int u) -> uint32_t {
       int o;
       if (wrap == 0) o = (lr * SW + c) * 64;
-      else if (wrap < 0) o = c < 2 ? (lr * 2 + c) * 64 : SR_MAX * 2 * 64 + (lr * 18 + c - 2) * 64;
-      else o = c < 18 ? (lr * 18 + c) * 64 : SR_MAX * 18 * 64 + (lr * 2 + c - 18) * 64;
+      else if (wrap < 0) o = c < 2 ? (lr * 2 + c) * 64 : SR_MAX * 2 * 64 + (lr * (SW - 2) + c - 2) * 64;
+      else o = c < SW - 2 ? (lr * (SW - 2) + c) * 64 : SR_MAX * (SW - 2) * 64 + (lr * 2 + c - (SW - 2)) * 64;
       o += u * 16;
       return (uint32_t)(o ^ (((o >> 7) & 3) << 4));
     };
@@ -563,11 +651,11 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
     int kst = 0, kpar = 0;   // K/V ring position and its use parity
 
     auto vec = [&](int j) -> const float4* { return reinterpret_cast<const float4*>(smem + OFF_VEC + (j & 1) * VEC_BYTES); };
-    // QKV epilogue: + bias, bf16. The 128 x 384 tile is staged in shared memory
+    // QKV epilogue: + bias, bf16. The TP x 384 tile is staged in shared memory
     // (chunk 0 in the A operand, chunks 1 and 2 in the GELU region, all free
     // once the QKV MMAs are done) in the operand layout, then written to the
-    // global qkv array of block buffer `buf` in whole rows: the patch's 16
-    // tokens of a latitude are 12 KB of consecutive memory.
+    // global qkv array of block buffer `buf` in whole rows: the patch's TW
+    // tokens of a latitude are consecutive in memory.
     auto qkv_epilogue = [&](const float4* vb, int buf) {
       ok = warp_wait(&mma_done, (uint32_t)(md++) & 1u, &abort_flag) && ok;
       if (!ok) abort_flag = 1;
@@ -575,17 +663,17 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       const float4* bq = vb + V_BQKV / 4;
 #pragma unroll 1
       for (int c = 0; c < 3; ++c) {
-        uint8_t* stg = smem + (c == 0 ? OFF_A : OFF_H + (c - 1) * CHUNK) + hf * SLICE + r * 128;
+        uint8_t* stg = smem + (c == 0 ? OFF_A : OFF_H + (c - 1) * CHUNK) + pl.hf * SLICE + pl.tr * 128;
 #pragma unroll 1
-        for (int sub = 0; sub < 2; ++sub) {
-          const int col = 128 * c + 64 * hf + 32 * sub;
-          float acc[32];
-          tmem_ld32(tmem + T_ACC1 + (uint32_t)col + lane_off, acc);
+        for (int sub = 0; sub < NC; sub += NS) {
+          const int col = 128 * c + pl.c0 + sub;
+          float acc[NS];
+          tmem_ld<NS>(tmem + T_ACC1 + (uint32_t)col + lane_off, acc);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
+          for (int k = 0; k < NS / 8; ++k) {
             const float4 b0 = bq[(col >> 2) + 2 * k], b1 = bq[(col >> 2) + 2 * k + 1];
-            const int j = 8 * k;
-            *reinterpret_cast<uint4*>(stg + (((4 * sub + k) ^ (r & 7)) << 4)) =
+            const int j = 8 * k, u = ((NC * pl.copy + sub) >> 3) + k;
+            *reinterpret_cast<uint4*>(stg + ((u ^ (pl.tr & 7)) << 4)) =
                 make_uint4(pack_bf16(acc[j] + b0.x, acc[j + 1] + b0.y), pack_bf16(acc[j + 2] + b0.z, acc[j + 3] + b0.w),
                            pack_bf16(acc[j + 4] + b1.x, acc[j + 5] + b1.y), pack_bf16(acc[j + 6] + b1.z, acc[j + 7] + b1.w));
           }
@@ -596,11 +684,11 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       // 16-byte piece p (0 .. 47) of tile row rr, consecutive threads along a row
       bf16* dst = a.qkv + ((long)buf * a.G + g) * N * QKV;
 #pragma unroll 4
-      for (int it = threadIdx.x; it < 128 * 48; it += 256) {
+      for (int it = threadIdx.x; it < TP * 48; it += 256) {
         const int rr = it / 48, p = it - rr * 48;
         const int c = p >> 4, sl = (p >> 3) & 1, u = p & 7;
         const uint8_t* src = smem + (c == 0 ? OFF_A : OFF_H + (c - 1) * CHUNK) + sl * SLICE + rr * 128 + ((u ^ (rr & 7)) << 4);
-        const int tok = (d * a.H + h0 + (rr >> 4)) * a.W + w0 + (rr & 15);
+        const int tok = (d * a.H + h0 + rr / TW) * a.W + w0 + rr % TW;
         *reinterpret_cast<uint4*>(dst + (long)tok * QKV + 8 * p) = *reinterpret_cast<const uint4*>(src);
       }
     };
@@ -614,7 +702,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
     {
       const float4* src = reinterpret_cast<const float4*>(xg);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
+      for (int q = 0; q < NC / 4; ++q) {
         const float4 x = src[q];
         v[4 * q] = x.x;
         v[4 * q + 1] = x.y;
@@ -622,15 +710,15 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         v[4 * q + 3] = x.w;
       }
 #pragma unroll
-      for (int sub = 0; sub < 2; ++sub) {
-        float t[32];
+      for (int sub = 0; sub < NC; sub += NS) {
+        float t[NS];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) t[j] = v[32 * sub + j];
-        tmem_st32(tmem + T_X + (uint32_t)(64 * hf + 32 * sub) + lane_off, t);
+        for (int j = 0; j < NS; ++j) t[j] = v[sub + j];
+        tmem_st<NS>(tmem + T_X + (uint32_t)(pl.c0 + sub) + lane_off, t);
       }
       tmem_wait_st();
       ok = warp_wait(&vec_full[0], 0u, &abort_flag) && ok;
-      layernorm_to_a(smem, v, r, hf, vec(0) + V_LN1G / 4, vec(0) + V_LN1B / 4, a.eps);
+      layernorm_to_a<TP>(smem, v, pl, vec(0) + V_LN1G / 4, vec(0) + V_LN1B / 4, a.eps);
       a_ready();
       qkv_epilogue(vec(0), 0);
     }
@@ -657,10 +745,10 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         };
         float o[4][4], l0 = 0.f, l1 = 0.f, m0 = -INFINITY, m1 = -INFINITY;
         uint32_t qa[2][4], qn[2][4];
-        load_q(0, qn);
+        load_q(hs * NH, qn);
 #pragma unroll 1
         for (int s = 0; s < steps; ++s) {
-          const int h = s / a.kd, lv = s % a.kd;
+          const int hi = s / a.kd, lv = s - hi * a.kd, h = hs * NH + hi;
           ok = warp_wait(&kv_full[kst], (uint32_t)kpar, &abort_flag) && ok;
           if (!ok) abort_flag = 1;
           if (lv == 0) {
@@ -668,13 +756,13 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
             for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
               for (int e = 0; e < 4; ++e) qa[kk][e] = qn[kk][e];
-            if (h + 1 < 4) load_q(h + 1, qn);   // the next head's queries, in flight during this head
+            if (hi + 1 < NH) load_q(h + 1, qn);   // the next head's queries, in flight during this head
 #pragma unroll
             for (int nb8 = 0; nb8 < 4; ++nb8) o[nb8][0] = o[nb8][1] = o[nb8][2] = o[nb8][3] = 0.f;
             l0 = l1 = 0.f;
             m0 = m1 = -INFINITY;
           }
-          const uint32_t kb = sbase + kv_stage_off(kst);
+          const uint32_t kb = sbase + CF::kv_stage_off(kst) + hs * 2 * KV_SLAB;
           // S = Q K^T over the 8 x 8 key rectangle (8 n8 blocks, one per rectangle row)
           float sc[8][4];
 #pragma unroll
@@ -752,8 +840,13 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
 #pragma unroll
             for (int nb8 = 0; nb8 < 4; ++nb8) {
               const int ch = h * DH + 8 * nb8 + 2 * t4;
-              *reinterpret_cast<uint32_t*>(smem + OFF_A + op_off(ri0, ch)) = pack_bf16(o[nb8][0] * i0, o[nb8][1] * i0);
-              *reinterpret_cast<uint32_t*>(smem + OFF_A + op_off(ri1, ch)) = pack_bf16(o[nb8][2] * i1, o[nb8][3] * i1);
+              const uint32_t p0 = pack_bf16(o[nb8][0] * i0, o[nb8][1] * i0);
+              const uint32_t p1 = pack_bf16(o[nb8][2] * i1, o[nb8][3] * i1);
+#pragma unroll
+              for (int c = 0; c < NCP; ++c) {
+                *reinterpret_cast<uint32_t*>(smem + OFF_A + op_off(c * TP + ri0, ch)) = p0;
+                *reinterpret_cast<uint32_t*>(smem + OFF_A + op_off(c * TP + ri1, ch)) = p1;
+              }
             }
           }
         }
@@ -763,9 +856,9 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       ok = warp_wait(&mma_done, (uint32_t)(md++) & 1u, &abort_flag) && ok;
       if (!ok) abort_flag = 1;
       tc_fence_after();
-      residual_add(tmem, lane_off, T_PROJ, hf, vb + V_BO / 4, v);
+      residual_add<TP>(tmem, lane_off, T_PROJ, pl, vb + V_BO / 4, v);
       tc_fence_before();
-      layernorm_to_a(smem, v, r, hf, vb + V_LN2G / 4, vb + V_LN2B / 4, a.eps);
+      layernorm_to_a<TP>(smem, v, pl, vb + V_LN2G / 4, vb + V_LN2B / 4, a.eps);
       a_ready();
       // ------------------------------------------------ MLP: FC1 chunks -> GELU -> shared memory
 #pragma unroll 1
@@ -774,20 +867,20 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         ok = warp_wait(&acc1_full[b], (uint32_t)(j >> 1), &abort_flag) && ok;
         if (!ok) abort_flag = 1;
         tc_fence_after();
-        uint8_t* H = smem + OFF_H + b * CHUNK + hf * SLICE;
+        uint8_t* H = smem + OFF_H + b * CHUNK + pl.hf * SLICE + pl.tr * 128;
 #pragma unroll 1
-        for (int sub = 0; sub < 2; ++sub) {
-          const int c = 64 * hf + 32 * sub;
-          float acc[32];
-          tmem_ld32(tmem + T_ACC1 + (uint32_t)(128 * b + c) + lane_off, acc);
-          if (sub == 1) {
+        for (int sub = 0; sub < NC; sub += NS) {
+          const int c = pl.c0 + sub;
+          float acc[NS];
+          tmem_ld<NS>(tmem + T_ACC1 + (uint32_t)(128 * b + c) + lane_off, acc);
+          if (sub + NS == NC) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc1_empty[b]);
           }
           const float4* b1 = vb + (V_B1 + 128 * j + c) / 4;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
+          for (int q = 0; q < NS / 4; ++q) {
             const float4 bb = b1[q];
             acc[4 * q] += bb.x;
             acc[4 * q + 1] += bb.y;
@@ -795,18 +888,21 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
             acc[4 * q + 3] += bb.w;
           }
 #pragma unroll
-          for (int jj = 0; jj < 32; jj += 2) gelu_erf2(acc[jj], acc[jj + 1]);
+          for (int jj = 0; jj < NS; jj += 2) gelu_erf2(acc[jj], acc[jj + 1]);
           if (sub == 0 && j >= 2) {
             // this slot's previous chunk has been read by FC2
             ok = warp_wait(&h_empty[b], 0u, &abort_flag) && ok;
             if (!ok) abort_flag = 1;
           }
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
+          for (int k = 0; k < NS / 8; ++k) {
             uint32_t w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) w[e] = pack_bf16(acc[8 * k + 2 * e], acc[8 * k + 2 * e + 1]);
-            *reinterpret_cast<uint4*>(H + r * 128 + (((4 * sub + k) ^ (r & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+            const int u = ((NC * pl.copy + sub) >> 3) + k;
+#pragma unroll
+            for (int cp = 0; cp < NCP; ++cp)
+              *reinterpret_cast<uint4*>(H + cp * TP * 128 + ((u ^ (pl.tr & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
         fence_async_smem();
@@ -817,7 +913,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       ok = warp_wait(&mma_done, (uint32_t)(md++) & 1u, &abort_flag) && ok;
       if (!ok) abort_flag = 1;
       tc_fence_after();
-      residual_add(tmem, lane_off, T_ACC2, hf, vb + V_B2 / 4, v);
+      residual_add<TP>(tmem, lane_off, T_ACC2, pl, vb + V_B2 / 4, v);
       tc_fence_before();
       // block i's vectors are no longer needed: their slot may take block i + 2's
       __syncwarp();
@@ -827,7 +923,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         ok = warp_wait(&vec_full[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1u, &abort_flag) && ok;
         if (!ok) abort_flag = 1;
         const float4* vn = vec(i + 1);
-        layernorm_to_a(smem, v, r, hf, vn + V_LN1G / 4, vn + V_LN1B / 4, a.eps);
+        layernorm_to_a<TP>(smem, v, pl, vn + V_LN1G / 4, vn + V_LN1B / 4, a.eps);
         a_ready();
         qkv_epilogue(vn, (i + 1) & 1);
         run = latent_barrier(a.bar + g, (++epoch) * (unsigned)a.T, warp, lane, &abort_flag);
@@ -838,7 +934,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         if (run) {
           float4* dst = reinterpret_cast<float4*>(xg);
 #pragma unroll
-          for (int q = 0; q < 16; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          for (int q = 0; q < NC / 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
       }
     }
@@ -850,6 +946,8 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
 
   tc_fence_before();
   __syncthreads();
+  // a hint for the host's choice of patch sizes: latent 0's first patch is through
+  if (a.done && blockIdx.x == 0 && threadIdx.x == 0) *(volatile unsigned int*)a.done = a.seq;
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
@@ -879,38 +977,51 @@ wm_status launch_swizzle_chunk(const float* W, int ld, __nv_bfloat16* out, cudaS
   return WM_OK;
 }
 
-int rollout_small_capacity() {
-  static int cap = -1;
+namespace rs {
+
+template <int TP>
+int capacity() {
+  static std::atomic<int> cap{-1};
   if (cap >= 0) return cap;
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaFuncSetAttribute(rs::rollout_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::SMEM) !=
+  if (cudaFuncSetAttribute(rollout_small_kernel<TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<TP>::SMEM) !=
       cudaSuccess)
     return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, rs::rollout_small_kernel, rs::THREADS, rs::SMEM) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, rollout_small_kernel<TP>, THREADS, Cfg<TP>::SMEM) !=
       cudaSuccess)
     return 0;
   cap = per * sms;
   return cap;
 }
 
-wm_status launch_rollout_small(const RolloutSmallArgs& a, cudaStream_t s) {
-  const int grid = a.G * a.T;
-  if (a.G < 1 || a.G > kRolloutSmallMaxLatents || grid > rollout_small_capacity())
-    return fail(WM_ERR_INVALID_ARG, "small-latent rollout kernel: too many tiles for one cooperative launch");
+template <int TP>
+wm_status launch(const RolloutSmallArgs& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(rs::THREADS);
-  cfg.dynamicSmemBytes = rs::SMEM;
+  cfg.gridDim = dim3((unsigned)(a.G * a.T));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = Cfg<TP>::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  WM_CUDA(cudaLaunchKernelEx(&cfg, rs::rollout_small_kernel, a));
+  WM_CUDA(cudaLaunchKernelEx(&cfg, rollout_small_kernel<TP>, a));
   return WM_OK;
+}
+
+}  // namespace rs
+
+int rollout_small_capacity(int tokens) {
+  return tokens == 128 ? rs::capacity<128>() : tokens == 64 ? rs::capacity<64>() : tokens == 32 ? rs::capacity<32>() : 0;
+}
+
+wm_status launch_rollout_small(const RolloutSmallArgs& a, cudaStream_t s) {
+  if (a.G < 1 || a.G > kRolloutSmallMaxLatents || a.G * a.T > rollout_small_capacity(a.tokens))
+    return fail(WM_ERR_INVALID_ARG, "small-latent rollout kernel: too many tiles for one cooperative launch");
+  return a.tokens == 128 ? rs::launch<128>(a, s) : a.tokens == 64 ? rs::launch<64>(a, s) : rs::launch<32>(a, s);
 }
 
 }  // namespace wm

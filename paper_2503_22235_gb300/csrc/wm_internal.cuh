@@ -319,10 +319,14 @@ struct RolloutBlock {
                             // ln2_b [128 each] b1[512] b2[128]
 };
 struct RolloutSmallArgs {
-  CUtensorMap tm_kv[3];      // make_tmap_kv_slab over qkv ([2 G D][H][W][384]): 20, 18, 2 longitudes x 12 latitudes
+  CUtensorMap tm_kv[3];      // make_tmap_kv_slab over qkv ([2 G D][H][W][384]): tokens / 8 + 4, tokens / 8 + 2 and 2
+                             // longitudes x 12 latitudes
   const RolloutBlock* blk;   // device array: the six-hour blocks, then the one-hour blocks
   int L6, L1;                // blocks per processor
-  int G, T;                  // latents; CTAs (8 x 16-token patches) per latent
+  int G, T;                  // latents; CTAs (patches) per latent
+  unsigned int* done;        // host word set to seq when the launch ends (nullptr: none)
+  unsigned int seq;
+  int tokens;                // per patch: 128, 64 or 32 (8 latitudes x 16, 8 or 4 longitudes); results do not depend on it
   int D, H, W, kd, kh, kw;   // H % 8 == 0, W % 16 == 0, W >= 32, kh <= 5, kw <= 5, periodic longitude
   float* x[kRolloutSmallMaxLatents];     // fp32 latents [D*H*W, 128], updated in place
   int n6[kRolloutSmallMaxLatents];       // six-hour steps per latent (then n1 one-hour steps)
@@ -332,8 +336,8 @@ struct RolloutSmallArgs {
   int* status;               // device status word
   float eps, scale_log2;     // LayerNorm epsilon; log2(e) / sqrt(32)
 };
-// CTAs the device can hold at once for the rollout kernel (0 when unknown).
-int rollout_small_capacity();
+// CTAs of patches of `tokens` tokens the device can hold at once for the rollout kernel (0 when unknown).
+int rollout_small_capacity(int tokens);
 wm_status launch_rollout_small(const RolloutSmallArgs& a, cudaStream_t s);
 // W[n][k] (row stride ld floats), n, k < 128, to one bf16 chunk of the layout above.
 wm_status launch_swizzle_chunk(const float* W, int ld, __nv_bfloat16* out, cudaStream_t s);
