@@ -791,6 +791,87 @@ struct RolloutTraffic {
   int peak() const { return std::max(1, *std::max_element(recent, recent + 8)); }
 } g_rollout_traffic;
 
+// Tokens of a patch for G latents in one launch: fewer tokens a CTA shorten
+// every phase of a block, so a launch takes the smallest patches whose CTAs
+// are all on the device at once, with as many launches beside it as other
+// streams were lately seen to have in flight (launches that fill the chip
+// would take turns). us per block of 4 x 24 x 48: one latent 33.3 with
+// 128-token patches, 16.9 with 32; two 33.3, and 22.0 with 64. Four contexts
+// on four streams, one 64-block rollout each: 2213 us with 128, 4288 with 32.
+int rollout_small_tokens(const wm_config& c, int G, int streams) {
+  int tokens = 128;
+  for (int t : {64, 32})
+    if (streams * G * c.D * (c.H / 8) * (c.W / (t / 8)) <= wm::rollout_small_capacity(t)) tokens = t;
+  return tokens;
+}
+
+// One launch of an uneven batch: the latents and the steps each advances.
+struct RolloutPart {
+  std::vector<int> idx, n6, n1;
+};
+
+// Launches of up to G latents that bring latent i n6[i] six-hour, then n1[i]
+// one-hour steps forward. `cut` false: the longest rollouts first, each in one
+// launch, so a launch lasts as long as its longest and its other places idle
+// behind the shorter ones. `cut` true: rollouts are cut at steps (the
+// residual is FP32 in memory and in the kernel, so the bits are the same).
+// While more than G wait, the G longest run until the first of those that wait
+// could no longer end with the rest (whole time: the mean load of G places or
+// the longest rollout), or one of them ends; once all are in, they run until
+// so few are left that these take smaller patches. Eight latents of 4 x 24 x
+// 48 with lead times drawn evenly up to 48 h, three draws: 3342, 3384, 3438 us
+// in two launches; 2725, 2855, 2996 us in four to six.
+std::vector<RolloutPart> rollout_small_plan(const wm_config& c, int G, std::vector<int> n6, std::vector<int> n1,
+                                            bool cut, int streams) {
+  const int L6 = c.blocks_p6, L1 = c.blocks_p1;
+  auto left = [&](int i) { return n6[i] * L6 + n1[i] * L1; };
+  std::vector<int> live(n6.size());
+  for (size_t i = 0; i < live.size(); ++i) live[i] = (int)i;
+  std::vector<RolloutPart> parts;
+  while (true) {
+    live.erase(std::remove_if(live.begin(), live.end(), [&](int i) { return n6[i] + n1[i] == 0; }), live.end());
+    if (live.empty()) return parts;
+    std::stable_sort(live.begin(), live.end(), [&](int p, int q) { return left(p) > left(q); });
+    const int g = std::min((int)live.size(), G);
+    int run = left(live[0]);   // blocks of this launch
+    if (cut && (int)live.size() > G) {
+      long sum = 0;
+      for (int i : live) sum += left(i);
+      const int whole = std::max((int)((sum + G - 1) / G), run);
+      run = std::min(left(live[G - 1]), std::max(L6, whole - left(live[G])));
+    } else if (cut) {
+      int k = g - 1;
+      while (k > 0 && rollout_small_tokens(c, k, streams) == rollout_small_tokens(c, g, streams)) --k;
+      if (k > 0) run = left(live[k]);
+    }
+    RolloutPart p;
+    for (int j = 0; j < g; ++j) {
+      const int i = live[j];
+      int s6 = std::min(n6[i], run / L6);
+      int s1 = s6 == n6[i] ? std::min(n1[i], (run - s6 * L6) / L1) : 0;
+      if (s6 + s1 == 0) (n6[i] > 0 ? s6 : s1) = 1;   // a step at least
+      p.idx.push_back(i);
+      p.n6.push_back(s6);
+      p.n1.push_back(s1);
+      n6[i] -= s6;
+      n1[i] -= s1;
+    }
+    parts.push_back(p);
+  }
+}
+
+// us of a plan: measured per block and launch on 4 x 24 x 48.
+double rollout_small_time(const wm_config& c, const std::vector<RolloutPart>& parts, int streams) {
+  double us = 0;
+  for (const RolloutPart& p : parts) {
+    int most = 0;
+    for (size_t j = 0; j < p.idx.size(); ++j) most = std::max(most, p.n6[j] * c.blocks_p6 + p.n1[j] * c.blocks_p1);
+    const int t = rollout_small_tokens(c, (int)p.idx.size(), streams);
+    us += 7.0 + most * (t == 32 ? 16.9 : t == 64 ? 22.0 : 33.6);
+  }
+  return us;
+}
+
 // Once per context: every block's weights as 12 swizzled bf16 chunks and the
 // per-block table the kernel reads.
 wm_status prepare_rollout_small(wm_ctx* ctx) {
@@ -856,13 +937,6 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   a.L6 = c.blocks_p6;
   a.L1 = c.blocks_p1;
   a.G = G;
-  // Fewer tokens a CTA shorten every phase of a block, so a launch takes the
-  // smallest patches whose CTAs are all on the device at once, with as many
-  // launches beside it as other streams were lately seen to have in flight
-  // (launches that fill the chip would take turns). us per block of
-  // 4 x 24 x 48: one latent 33.3 with 128-token patches, 16.9 with 32; two
-  // 33.3, and 22.0 with 64. Four contexts on four streams, one 64-block
-  // rollout each: 2213 us with 128, 4288 with 32.
   const bool counted = cap == cudaStreamCaptureStatusNone;   // a captured launch runs later, any number of times
   const int streams = counted ? g_rollout_traffic.enter(ctx, s, &a.seq) : g_rollout_traffic.seen();
   if (counted) a.done = ctx->h_rs_done;
@@ -870,9 +944,7 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
     wm_ctx* ctx;
     ~Undo() { if (ctx) g_rollout_traffic.undo(ctx); }
   } undo{counted ? ctx : nullptr};
-  a.tokens = 128;
-  for (int t : {64, 32})
-    if (streams * G * c.D * (c.H / 8) * (c.W / (t / 8)) <= wm::rollout_small_capacity(t)) a.tokens = t;
+  a.tokens = rollout_small_tokens(c, G, streams);
   a.T = c.D * (c.H / 8) * (c.W / (a.tokens / 8));
   a.D = c.D; a.H = c.H; a.W = c.W; a.kd = c.kd; a.kh = c.kh; a.kw = c.kw;
   for (int i = 0; i < G; ++i) {
@@ -1398,23 +1470,16 @@ wm_status wm_rollout_batch(wm_ctx* ctx, float* const* latents, const int* lead_h
   const int G = rollout_small_group(ctx, n);
   if (G > 0) {
     // narrow latent: launches of up to G latents with their own schedules,
-    // longest rollouts together, read and written in place (no gather)
-    std::vector<int> order;
-    for (int i = 0; i < n; ++i)
-      if (n6[i] + n1[i] > 0) order.push_back(i);
-    const int L6 = ctx->cfg.blocks_p6, L1 = ctx->cfg.blocks_p1;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int p, int q) { return n6[p] * L6 + n1[p] * L1 > n6[q] * L6 + n1[q] * L1; });
-    for (size_t i0 = 0; i0 < order.size(); i0 += G) {
-      const int g = (int)std::min(order.size() - i0, (size_t)G);
-      std::vector<float*> xs(g);
-      std::vector<int> a6(g), a1(g);
-      for (int i = 0; i < g; ++i) {
-        xs[i] = latents[order[i0 + i]];
-        a6[i] = n6[order[i0 + i]];
-        a1[i] = n1[order[i0 + i]];
-      }
-      WM_TRY(rollout_small(ctx, xs.data(), a6.data(), a1.data(), g, (cudaStream_t)stream));
+    // read and written in place (no gather)
+    const wm_config& c = ctx->cfg;
+    const int streams = g_rollout_traffic.seen();
+    std::vector<RolloutPart> parts = rollout_small_plan(c, G, n6, n1, false, streams);
+    std::vector<RolloutPart> cut = rollout_small_plan(c, G, n6, n1, true, streams);
+    if (rollout_small_time(c, cut, streams) < rollout_small_time(c, parts, streams)) parts.swap(cut);
+    for (const RolloutPart& p : parts) {
+      std::vector<float*> xs;
+      for (int i : p.idx) xs.push_back(latents[i]);
+      WM_TRY(rollout_small(ctx, xs.data(), p.n6.data(), p.n1.data(), (int)xs.size(), (cudaStream_t)stream));
     }
     return WM_OK;
   }
