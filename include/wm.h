@@ -351,7 +351,7 @@ wm_status wm_fp8_scales(wm_ctx* ctx, int which, int block, float* out);
  * 1 = 128-column tiles, 2 = 256-column tiles, 3 = 256 x 256 tiles on CTA pairs
  * (cta_group::2; shapes with N % 256 != 0 keep single-CTA tiles), 4 = 64-column
  * tiles (N % 64 == 0). Applies to every BF16 / FP8-MLP block GEMM launched or
- * captured afterwards and to wm_op_linear (BF16; pairs for epilogue 0 only).
+ * captured afterwards and to wm_op_linear (BF16; pairs for epilogues 0 and 1).
  * Results are the same function of the inputs in every mode up to
  * accumulation rounding; the tile width also sets how the LayerNorm
  * statistics partials are split (two per tile). WM_ERR_INVALID_ARG for a

@@ -291,6 +291,17 @@ int pick_bn(long M, int N) {
   return 128;
 }
 
+// Linear layers alone (the block's GEMMs are tuned): 256 x 256 tiles on CTA
+// pairs where they fill every pair twice and the K loop is long enough to
+// matter, us for 256-column tiles -> pairs: 40,000 x 1536 x 768 72 -> 61 (GELU
+// 75 -> 70), 20,475 x 768 x 3072 74 -> 64, 145,800 x 3072 x 768 467 -> 402 (533
+// -> 493); but 40,000 x 1536 x 128 31 -> 35, and 9000 x 768 x 3072 (108 tiles) 35
+// -> 35. The bits are the same.
+bool pick_pair(long M, int N, int K, int epi) {
+  return (epi == wm::EPI_STORE || epi == wm::EPI_GELU) && K >= 768 &&
+         ((M + 255) / 256) * (N / 256) >= wm::num_sms() && wm::gemm_pairs_fit();
+}
+
 // ---- GEMM tile autotuner
 // Tile width BN (64, 128 or 256 output columns; 256 also as 256 x 256 tiles on
 // CTA pairs) and, for the residual epilogue, one or two staging tiles,
@@ -1694,7 +1705,8 @@ wm_status wm_op_linear(const void* A, const void* W, const float* bias, void* ou
   wm::GemmArgs a;
   const int ov = g_gemm_override.load();
   a.bn = ov == 1 ? 128 : ov == 4 ? 64 : (ov >= 2 && N % 256 == 0) ? 256 : pick_bn(M, N);
-  a.pair = ov == 3 && a.bn == 256 && epilogue == wm::EPI_STORE;
+  a.pair = a.bn == 256 && (ov == 3 ? epilogue == wm::EPI_STORE || epilogue == wm::EPI_GELU
+                                   : ov == 0 && pick_pair(M, N, K, epilogue));
   const bool out_f32 = epilogue == wm::EPI_RESID_F32 || epilogue == wm::EPI_STORE_F32;
   if (!wm::make_tmap_bf16(&a.tmA, A, (uint64_t)M, (uint64_t)K, 128) ||
       !wm::make_tmap_bf16(&a.tmB, W, (uint64_t)N, (uint64_t)K, (uint32_t)(a.pair ? 128 : a.bn)) ||

@@ -10,9 +10,10 @@
 //              into one of two TMEM accumulators; tcgen05.commit frees the
 //              smem stage and, after the last k-slice, hands the accumulator
 //              to the epilogue.
-//   warps 2-9  epilogue: tcgen05.ld (32x32b) rows out of TMEM, add bias, then
-//              bf16 store, GELU + bf16 store, or FP32 residual add, while the
-//              MMA warp already fills the other accumulator.
+//   warps 2-9  epilogue (2-17 where it evaluates GELU): tcgen05.ld (32x32b)
+//              rows out of TMEM, add bias, then bf16 store, GELU + bf16 store,
+//              or FP32 residual add, while the MMA warp already fills the
+//              other accumulator.
 // Pair mode (BN = 256, PAIR): a cluster of two CTAs on two SMs computes a
 // 256 x 256 tile with tcgen05.mma.cta_group::2 (M = 256). Each CTA loads its
 // own 128 A rows and its own 128 of the tile's 256 W rows, so each SM's
@@ -39,6 +40,19 @@ constexpr int BKB = 128;               // bytes per k-slice row (bf16: 64 elemen
 constexpr int NUM_EPI_WARPS = 8;
 constexpr int THREADS = 32 * (2 + NUM_EPI_WARPS);
 
+// Epilogue warps. GELU is some 20 instructions a column pair in dependent
+// chains: eight warps (two a scheduler) leave the issue slots 43 % busy and
+// the epilogue slower than the MMAs of its tile, sixteen hide the chains.
+// 145,800 x 3072 x 768 on pairs, random operands: 521 us with eight, 503 with
+// sixteen; zeros (nothing held back by power): 394, 362.
+// (The residual epilogue keeps eight: its row statistics follow the columns of
+// half a tile in order; the plain stores are not bound by it; a 64-column
+// tile has only two 32-column chunks a row.)
+__host__ __device__ constexpr int epi_warps(int bn, int epi) {
+  return (epi == EPI_GELU || epi == EPI_GELU_F8 || epi == EPI_LNF_GELU) && bn >= 128 ? 16 : NUM_EPI_WARPS;
+}
+__host__ __device__ constexpr int gemm_threads(int bn, int epi) { return 32 * (2 + epi_warps(bn, epi)); }
+
 // DUAL: a second (bf16) staging tile per epilogue warp; PAIR: this CTA holds half of the W tile
 template <int BN, bool DUAL = false, bool PAIR = false>
 struct Cfg {
@@ -46,7 +60,7 @@ struct Cfg {
   static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BKB;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = PAIR ? (DUAL ? 5 : 6) : (BN >= 256) ? (DUAL ? 3 : 4) : (DUAL ? 5 : 6);
-  static constexpr int EPI_STRIDE = DUAL ? 6144 : 4096;     // per epilogue warp: 32x32 fp32 (+ 32x32 bf16)
+  static constexpr int EPI_STRIDE = DUAL ? 6144 : 4096;     // per epilogue warp of 8: 32x32 fp32 (+ 32x32 bf16)
   static constexpr int EPI_BYTES = NUM_EPI_WARPS * EPI_STRIDE;
   static constexpr int SMEM = STAGES * STAGE_BYTES + EPI_BYTES + 1024;   // + alignment slack
   static constexpr int TMEM_COLS = 2 * BN;                   // two accumulators
@@ -130,7 +144,7 @@ __device__ __forceinline__ void stage_row(uint8_t* buf, const float (&x)[32], in
 }
 
 template <int BN, int EPI, bool F8, bool DUAL = false, bool PAIR = false>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(gemm_threads(BN, EPI), 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2, int M,
                         int N, int K, const EpiArgs e, int* __restrict__ status) {
@@ -143,6 +157,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   static_assert(!PAIR || BN == 256, "pair tiles are 256 x 256");
   constexpr int TM = PAIR ? 2 * BM : BM;  // output rows per tile (of the CTA pair)
   constexpr int STAGES = CF::STAGES;
+  constexpr int NEPI = epi_warps(BN, EPI);
+  static_assert(NEPI == 8 || !DUAL, "16 epilogue warps share the staging tiles of 8");
+  constexpr int EPI_STRIDE = CF::EPI_STRIDE * NUM_EPI_WARPS / NEPI;
+  constexpr int EPI_COLS = BN / (NEPI / 4);   // columns of one epilogue warp
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STAGES];
   __shared__ __align__(8) uint64_t empty_bar[STAGES];
@@ -154,7 +172,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int num_n = (N + BN - 1) / BN;
   const int num_tiles = ((M + TM - 1) / TM) * num_n;
   const int nk = (K + BKE - 1) / BKE;
@@ -171,7 +189,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf_bar[b], 1);
-      mbar_init(&acce_bar[b], PAIR ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS);
+      mbar_init(&acce_bar[b], PAIR ? 2 * NEPI : NEPI);
     }
     mbar_init(&drain_bar, 1);
     abort_flag = 0;
@@ -249,43 +267,63 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp == 1) {
+    // The whole warp walks the loop and one elected lane issues: with the loop
+    // inside one lane's branch, its addresses and waits took as long as the
+    // MMAs of a slice (512 clocks) and the tensor pipe idled between slices:
+    // 145,800 x 3072 x 768 on pairs, bf16 store, zeros: 404 -> 344 us, without
+    // loads and epilogue 342 -> 289 (1 / 1.03 of the MMA rate); random
+    // operands, where power sets the clock: 480 -> 441 in a long run.
     // (the odd CTA of a pair issues nothing here: the even CTA's thread issues the pair's MMAs)
-    if (lane == 0 && !(PAIR && rank != 0)) {
+    if (!(PAIR && rank != 0)) {
       // ------------------------------------------------------ MMA issuer
       constexpr uint32_t idesc = F8 ? idesc_e4m3(TM, BN) : idesc_bf16(TM, BN);
+      const bool leader = elect_one();
       int stage = 0;
       uint32_t phase = 0;
-      bool ok = true;
+      bool ok = true, ready = false;
       int it = 0;
       for (int tile = unit; tile < num_tiles && ok; tile += nunits, ++it) {
         const int buf = it & 1;
         const uint32_t acc_par = (uint32_t)(it >> 1) & 1u;
-        if (!(PAIR ? mbar_wait_cluster(&acce_bar[buf], acc_par ^ 1u, &abort_flag)
-                   : mbar_wait(&acce_bar[buf], acc_par ^ 1u, &abort_flag))) { ok = false; break; }
+        ok = __all_sync(0xffffffffu, PAIR ? mbar_wait_cluster(&acce_bar[buf], acc_par ^ 1u, &abort_flag)
+                                          : mbar_wait(&acce_bar[buf], acc_par ^ 1u, &abort_flag));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+#pragma unroll 1
         for (int kb = 0; kb < nk; ++kb) {
-          if (!(PAIR ? mbar_wait_cluster(&full_bar[stage], phase, &abort_flag)
-                     : mbar_wait(&full_bar[stage], phase, &abort_flag))) { ok = false; break; }
+          if (!ready) {
+            ok = __all_sync(0xffffffffu, PAIR ? mbar_wait_cluster(&full_bar[stage], phase, &abort_flag)
+                                              : mbar_wait(&full_bar[stage], phase, &abort_flag));
+            if (!ok) break;
+          }
           tc_fence_after();
           const uint32_t sa = smem_base + stage * CF::STAGE_BYTES;
-          const uint64_t adesc = sw128_desc(sa), bdesc = sw128_desc(sa + CF::A_BYTES);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {   // 4 MMAs of 32 bytes of K (16 bf16 / 32 e4m3) per slice
-            if constexpr (F8)
-              umma_e4m3<PAIR>(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0);
-            else
-              umma_bf16<PAIR>(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0);
-          }
-          if constexpr (PAIR) umma_commit_pair(&empty_bar[stage], 0x3);
-          else umma_commit(&empty_bar[stage]);
+          const int cur = stage;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          // is the next slice there already? (asked before this slice's MMAs, whose issue hides the answer's latency)
+          ready = __all_sync(0xffffffffu, PAIR ? mbar_test_cluster(smem_u32(&full_bar[stage]), phase)
+                                               : mbar_test(smem_u32(&full_bar[stage]), phase));
+          if (leader) {
+            const uint64_t adesc = sw128_desc(sa), bdesc = sw128_desc(sa + CF::A_BYTES);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {   // 4 MMAs of 32 bytes of K (16 bf16 / 32 e4m3) per slice
+              if constexpr (F8)
+                umma_e4m3<PAIR>(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0);
+              else
+                umma_bf16<PAIR>(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb | k) != 0);
+            }
+            if constexpr (PAIR) umma_commit_pair(&empty_bar[cur], 0x3);
+            else umma_commit(&empty_bar[cur]);
+          }
         }
         if (!ok) break;
-        if constexpr (PAIR) umma_commit_pair(&accf_bar[buf], 0x3);
-        else umma_commit(&accf_bar[buf]);
+        if (leader) {
+          if constexpr (PAIR) umma_commit_pair(&accf_bar[buf], 0x3);
+          else umma_commit(&accf_bar[buf]);
+        }
       }
-      if (!ok) {
+      if (!ok && leader) {
         abort_flag = 1;
         atomicExch(status, (int)WM_ERR_TIMEOUT);
         // completes once every MMA issued above has finished
@@ -298,35 +336,28 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else {
     // -------------------------------------------------------- epilogue
     const int quarter = warp & 3;                 // TMEM lane quarter this warp may access
-    const int half = (warp - 2) >> 2;             // which half of the BN columns
-    uint8_t* ebuf = smem + STAGES * CF::STAGE_BYTES + (warp - 2) * CF::EPI_STRIDE;
+    const int half = (warp - 2) >> 2;             // which half (quarter, of 16 warps) of the BN columns
+    uint8_t* ebuf = smem + STAGES * CF::STAGE_BYTES + (warp - 2) * EPI_STRIDE;
     const uint32_t ebuf32 = smem_u32(ebuf);
     uint8_t* ebuf2 = ebuf + 4096;                 // EPI_RESID_LN: the bf16 copy's staging tile
     const uint32_t ebuf2_32 = ebuf32 + 4096;
     // Narrow outputs (bf16: 2 KB per 32 x 32 chunk, e4m3: 1 KB) alternate
-    // between two halves of the warp's 4 KB staging tile, so a chunk waits
-    // only for the store of the chunk two before it.
-    constexpr bool kPing = !kResLN && EPI != EPI_RESID_F32 && EPI != EPI_STORE_F32;
+    // between two places of the warp's staging tile where it holds two, so a
+    // chunk waits only for the store of the chunk two before it.
     constexpr int kChunkBytes = EPI == EPI_GELU_F8 ? 1024 : 2048;
+    constexpr bool kPing =
+        !kResLN && EPI != EPI_RESID_F32 && EPI != EPI_STORE_F32 && EPI_STRIDE >= 2 * kChunkBytes;
     uint32_t staged = 0;                          // chunks this warp has staged (all tiles)
     int it = 0;
     for (int tile = unit; tile < num_tiles; tile += nunits, ++it) {
       const int buf = it & 1;
       const uint32_t acc_par = (uint32_t)(it >> 1) & 1u;
-      if (!(PAIR ? mbar_wait_cluster(&accf_bar[buf], acc_par, &abort_flag)
-                 : mbar_wait(&accf_bar[buf], acc_par, &abort_flag))) {
-        abort_flag = 1;
-        atomicExch(status, (int)WM_ERR_TIMEOUT);
-        break;
-      }
-      tc_fence_after();
       const int m0 = (tile / num_n) * TM + (int)rank * BM, n0 = (tile % num_n) * BN;
       const int row0 = m0 + quarter * 32;
       const int m = row0 + lane;
-      const uint32_t tbase = tmem_base + (uint32_t)(buf * BN) + ((uint32_t)(quarter * 32) << 16);
-      const int c_begin = half * (BN / 2), c_end = (half + 1) * (BN / 2);
       // LayerNorm folded into this GEMM: merge the row's partial (mean, M2)
-      // pairs (equal counts K / np each) into its mean and 1/sqrt(var + eps)
+      // pairs (equal counts K / np each) into its mean and 1/sqrt(var + eps),
+      // before the wait for the accumulator
       float ln_mean = 0.f, ln_rstd = 0.f;
       if constexpr (kLNF) {
         if (m < M) {
@@ -344,6 +375,15 @@ __global__ void __launch_bounds__(THREADS, 1)
           ln_rstd = rsqrtf(m2 / (float)K + e.eps);
         }
       }
+      if (!(PAIR ? mbar_wait_cluster(&accf_bar[buf], acc_par, &abort_flag)
+                 : mbar_wait(&accf_bar[buf], acc_par, &abort_flag))) {
+        abort_flag = 1;
+        atomicExch(status, (int)WM_ERR_TIMEOUT);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t tbase = tmem_base + (uint32_t)(buf * BN) + ((uint32_t)(quarter * 32) << 16);
+      const int c_begin = half * EPI_COLS, c_end = (half + 1) * EPI_COLS;
       // residual epilogue with row statistics: running Welford (count, mean, M2)
       float wn = 0.f, wmean = 0.f, wm2 = 0.f;
       float4 xa[kResLN ? 8 : 1];
@@ -373,28 +413,24 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         const int n = n0 + c;
         if (row0 >= M || n >= N) continue;   // whole chunk outside the output (warp-uniform)
-        float lcs[kLNF ? 32 : 1], lbb[kLNF ? 32 : 1];
-        if constexpr (kLNF) {   // column vectors of this chunk (N % 32 == 0 here)
+        if constexpr (kLNF) {
+          // rstd (acc - mean colsum) + b', then GELU, two columns per instruction (N % 32 == 0 here)
+          const uint64_t nmean2 = pack_f2(-ln_mean, -ln_mean), rstd2 = pack_f2(ln_rstd, ln_rstd);
           const float4* c4 = reinterpret_cast<const float4*>(e.colsum + n);
           const float4* b4 = reinterpret_cast<const float4*>(bias + n);
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            const float4 a = __ldg(c4 + q), b = __ldg(b4 + q);
-            lcs[4 * q] = a.x; lcs[4 * q + 1] = a.y; lcs[4 * q + 2] = a.z; lcs[4 * q + 3] = a.w;
-            lbb[4 * q] = b.x; lbb[4 * q + 1] = b.y; lbb[4 * q + 2] = b.z; lbb[4 * q + 3] = b.w;
-          }
-        }
-        if constexpr (kLNF) {
-          // rstd (acc - mean colsum) + b', then GELU, two columns per instruction
-          const uint64_t nmean2 = pack_f2(-ln_mean, -ln_mean), rstd2 = pack_f2(ln_rstd, ln_rstd);
+            const float4 cs = __ldg(c4 + q), bb = __ldg(b4 + q);
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            float t0, t1;
-            fma_f2(t0, t1, lcs[j], lcs[j + 1], nmean2, pack_f2(v[j], v[j + 1]));
-            fma_f2(v[j], v[j + 1], t0, t1, rstd2, pack_f2(lbb[j], lbb[j + 1]));
-            if constexpr (EPI == EPI_LNF_GELU) gelu_erf2(v[j], v[j + 1]);
+            for (int h = 0; h < 2; ++h) {
+              const int j = 4 * q + 2 * h;
+              float t0, t1;
+              fma_f2(t0, t1, h ? cs.z : cs.x, h ? cs.w : cs.y, nmean2, pack_f2(v[j], v[j + 1]));
+              fma_f2(v[j], v[j + 1], t0, t1, rstd2, h ? pack_f2(bb.z, bb.w) : pack_f2(bb.x, bb.y));
+              if constexpr (EPI == EPI_LNF_GELU) gelu_erf2(v[j], v[j + 1]);
+            }
           }
-        } else if ((EPI == EPI_GELU || EPI == EPI_GELU_F8) && bias && n + 32 <= N) {
+        } else if ((EPI == EPI_GELU || EPI == EPI_GELU_F8 || EPI == EPI_STORE) && bias && n + 32 <= N) {
           // whole chunk with a bias: the same steps two columns per instruction
           const uint64_t alpha2 = pack_f2(alpha, alpha), oscale2 = pack_f2(out_scale, out_scale);
           const float4* b4 = reinterpret_cast<const float4*>(bias + n);
@@ -406,7 +442,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               const int j = 4 * q + 2 * h;
               if constexpr (F8) mul_f2(v[j], v[j + 1], alpha2);
               add_f2(v[j], v[j + 1], v[j], v[j + 1], h ? b.z : b.x, h ? b.w : b.y);
-              gelu_erf2(v[j], v[j + 1]);
+              if constexpr (EPI != EPI_STORE) gelu_erf2(v[j], v[j + 1]);
               if constexpr (EPI == EPI_GELU_F8) mul_f2(v[j], v[j + 1], oscale2);
             }
           }
@@ -534,7 +570,7 @@ static int pair_capacity() {
   if (cap < 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * num_sms());
-    cfg.blockDim = dim3(THREADS);
+    cfg.blockDim = dim3(gemm_threads(BN, EPI));
     cfg.dynamicSmemBytes = Cfg<BN, DUAL, true>::SMEM;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -579,10 +615,10 @@ static wm_status launch_one(const GemmArgs& a, cudaStream_t s) {
   e.out_scale = a.out_scale;
   e.rope = a.rope;
   if constexpr (PAIR)
-    WM_CUDA(launch_pdl_pairs(kern, dim3(grid), dim3(THREADS), CF::SMEM, s, a.pdl, a.tmA, a.tmB, a.tmC, a.tmC2, a.M, a.N,
+    WM_CUDA(launch_pdl_pairs(kern, dim3(grid), dim3(gemm_threads(BN, EPI)), CF::SMEM, s, a.pdl, a.tmA, a.tmB, a.tmC, a.tmC2, a.M, a.N,
                              a.K, e, device_status_word()));
   else
-    WM_CUDA(launch_pdl(kern, dim3(grid), dim3(THREADS), CF::SMEM, s, a.pdl, a.tmA, a.tmB, a.tmC, a.tmC2, a.M, a.N, a.K,
+    WM_CUDA(launch_pdl(kern, dim3(grid), dim3(gemm_threads(BN, EPI)), CF::SMEM, s, a.pdl, a.tmA, a.tmB, a.tmC, a.tmC2, a.M, a.N, a.K,
                        e, device_status_word()));
   WM_CUDA(cudaGetLastError());
   return WM_OK;
@@ -622,12 +658,13 @@ static wm_status set_attrs_bn() {
     chk(set_attr<BN, EPI_RESID_LN, true, false, true>());
     chk(set_attr<BN, EPI_RESID_LN, true, true, true>());
     chk(set_attr<BN, EPI_STORE, false, false, true>());
+    chk(set_attr<BN, EPI_GELU, false, false, true>());
   }
   return st;
 }
 
-// The processor block's epilogues on 256 x 256 pair tiles (and a plain bf16
-// store for the per-op tests).
+// The processor block's epilogues on 256 x 256 pair tiles, and the plain and
+// the GELU bf16 store of the linear layers.
 static wm_status launch_pair(const GemmArgs& a, cudaStream_t s) {
   const bool dual = a.dual >= 0 ? a.dual == 1 : a.K <= 1024;
   if (a.f8) {
@@ -641,6 +678,7 @@ static wm_status launch_pair(const GemmArgs& a, cudaStream_t s) {
   }
   switch (a.epi) {
     case EPI_STORE: return launch_one<256, EPI_STORE, false, false, true>(a, s);
+    case EPI_GELU: return launch_one<256, EPI_GELU, false, false, true>(a, s);
     case EPI_RESID_LN:
       return dual ? launch_one<256, EPI_RESID_LN, false, true, true>(a, s)
                   : launch_one<256, EPI_RESID_LN, false, false, true>(a, s);
@@ -1106,6 +1144,8 @@ wm_status launch_mlp_small(const MlpArgs& a, cudaStream_t s) {
     return fail(WM_ERR_INVALID_ARG, "fused MLP needs 16-byte aligned residual buffers");
   return tc::launch_mlp(a, s);
 }
+
+bool gemm_pairs_fit() { return tc::pair_capacity<256, EPI_STORE, false, false>() >= 1; }
 
 wm_status launch_gemm_tc(const GemmArgs& a, cudaStream_t s) {
   if (a.M <= 0 || a.N <= 0) return WM_OK;

@@ -280,6 +280,8 @@ struct GemmArgs {
 };
 // Rotate q and k in an fp32 qkv [M, 3C] (the FP32 plain path).
 wm_status launch_rope_f32(float* qkv, long M, const RopeArgs* rope_dev, const RopeArgs& rope_host, cudaStream_t s);
+// Whether two-CTA clusters of the pair GEMM fit on the device.
+bool gemm_pairs_fit();
 wm_status launch_gemm_tc(const GemmArgs& a, cudaStream_t s);
 
 // The small latent's MLP (C = 128, hidden 512) fused into one kernel: FC1 with
