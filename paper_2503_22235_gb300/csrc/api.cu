@@ -806,8 +806,8 @@ struct RolloutTraffic {
 // every phase of a block, so a launch takes the smallest patches whose CTAs
 // are all on the device at once, with as many launches beside it as other
 // streams were lately seen to have in flight (launches that fill the chip
-// would take turns). us per block of 4 x 24 x 48: one latent 33.3 with
-// 128-token patches, 16.9 with 32; two 33.3, and 22.0 with 64. Four contexts
+// would take turns). us per block of 4 x 24 x 48: one latent 32 with
+// 128-token patches, 16.5 with 32; two 32, and 21.9 with 64. Four contexts
 // on four streams, one 64-block rollout each: 2213 us with 128, 4288 with 32.
 int rollout_small_tokens(const wm_config& c, int G, int streams) {
   int tokens = 128;
@@ -831,7 +831,8 @@ struct RolloutPart {
 // the longest rollout), or one of them ends; once all are in, they run until
 // so few are left that these take smaller patches. Eight latents of 4 x 24 x
 // 48 with lead times drawn evenly up to 48 h, three draws: 3342, 3384, 3438 us
-// in two launches; 2725, 2855, 2996 us in four to six.
+// in two launches; 2725, 2855, 2996 us in four to six (2701 for the first with
+// the faster blocks).
 std::vector<RolloutPart> rollout_small_plan(const wm_config& c, int G, std::vector<int> n6, std::vector<int> n1,
                                             bool cut, int streams) {
   const int L6 = c.blocks_p6, L1 = c.blocks_p1;
@@ -878,7 +879,7 @@ double rollout_small_time(const wm_config& c, const std::vector<RolloutPart>& pa
     int most = 0;
     for (size_t j = 0; j < p.idx.size(); ++j) most = std::max(most, p.n6[j] * c.blocks_p6 + p.n1[j] * c.blocks_p1);
     const int t = rollout_small_tokens(c, (int)p.idx.size(), streams);
-    us += 7.0 + most * (t == 32 ? 16.9 : t == 64 ? 22.0 : 33.6);
+    us += 7.0 + most * (t == 32 ? 16.5 : t == 64 ? 21.9 : 32.0);
   }
   return us;
 }

@@ -22,7 +22,7 @@
 //              rows of A from shared memory (tensor copies, 128-byte swizzle)
 //              and write the three planes of A to tensor memory; W's planes
 //              lie in shared memory, 64-byte swizzle
-//   one thread issues the 12 tcgen05.mma of a slab (A from tensor memory, W
+//   one warp issues the 12 tcgen05.mma of a slab (A from tensor memory, W
 //              from shared memory; M = 128, N = BN, K = 16)
 //   one thread issues the tensor copies of A's slabs and W's planes
 //   summing    (eight warps) add a finished accumulator to their register
@@ -36,8 +36,11 @@
 // Weights that come ready as planes save the CTA two thirds of the splitting:
 // M = 145800, N = 768, K = 3072 took 4.8 ms with W split inside, 2.70 ms with
 // planes, 13.5 ms as FP32 FMAs on CUDA cores (51 TFLOP/s, now 255).
-// M = 20475, N = 1536, K = 384 with GELU: 559 us before, 149 now; M = 4608,
-// N = 512, K = 128 with GELU: 22.5 and 15.2 us.
+// M = 20475, N = 1536, K = 384 with GELU: 559 us before, 149 so; M = 4608,
+// N = 512, K = 128 with GELU: 22.5 and 15.2 us. The loop that issues the MMAs
+// inside one lane's branch left the tensor pipe idle between slabs; walked by
+// the whole warp, one elected lane issuing: 149 -> 136 us, a block of 145,800
+// tokens (C = 768) 13.41 -> 12.51 ms.
 //
 // NaN and infinity: a non-finite operand (or one that rounds up to infinity)
 // makes its second plane NaN, so every sum it enters comes out NaN. Operands
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int num_n = (N + BN - 1) / BN;
   const int num_tiles = ((M + BM - 1) / BM) * num_n;
   const int nk = (K + BK - 1) / BK;
@@ -346,8 +349,13 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
       }
     }
   } else if (warp == CF::MMA_WARP) {
-    if (lane == 0) {
+    {
       // ---------------------------------------------------------- MMA issue
+      // (the whole warp walks the loop, one elected lane issues)
+      const bool leader = elect_one();
+      auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+        return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag));
+      };
       constexpr uint32_t idesc = idesc_bf16(BM, BN);
       int stage = 0, buf = 0;
       uint32_t phase = 0, acc_phase = 0;
@@ -372,28 +380,31 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
           const bool two = kb + 1 < nk;   // slabs of this accumulator
           const int s0 = stage, s1 = stage + 1 == NST ? 0 : stage + 1, s2 = (stage + (two ? 2 : 1)) % NST;
           const uint32_t ph1 = s1 < s0 ? phase ^ 1u : phase, ph2 = s2 <= s0 ? phase ^ 1u : phase;
-          ok = mbar_wait(&acce_bar[buf], acc_phase ^ 1u, &abort_flag) &&
-               (ready || mbar_wait(&planes_full[s0], phase, &abort_flag));
+          ok = wait(&acce_bar[buf], acc_phase ^ 1u) && (ready || wait(&planes_full[s0], phase));
           if (!ok) break;
           tc_fence_after();
-          issue(s0, 2, 0u);
+          if (leader) issue(s0, 2, 0u);
           if (two) {
-            ok = mbar_wait(&planes_full[s1], ph1, &abort_flag);
+            ok = wait(&planes_full[s1], ph1);
             if (!ok) break;
             tc_fence_after();
-            issue(s1, 2, 1u);
+            if (leader) issue(s1, 2, 1u);
           }
-          issue(s0, 1, 1u);
-          if (two) issue(s1, 1, 1u);
+          if (leader) {
+            issue(s0, 1, 1u);
+            if (two) issue(s1, 1, 1u);
+          }
           // while the tensor core works: are the next accumulator's first planes there?
-          ready = mbar_try_wait(smem_u32(&planes_full[s2]), ph2);
-          issue(s0, 0, 1u);
-          umma_commit(&planes_empty[s0]);
-          if (two) {
-            issue(s1, 0, 1u);
-            umma_commit(&planes_empty[s1]);
+          ready = __all_sync(0xffffffffu, mbar_test(smem_u32(&planes_full[s2]), ph2));
+          if (leader) {
+            issue(s0, 0, 1u);
+            umma_commit(&planes_empty[s0]);
+            if (two) {
+              issue(s1, 0, 1u);
+              umma_commit(&planes_empty[s1]);
+            }
+            umma_commit(&accf_bar[buf]);
           }
-          umma_commit(&accf_bar[buf]);
           stage = s2;
           phase = ph2;
           if (++buf == NACC) {
@@ -402,7 +413,7 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
           }
         }
       }
-      if (!ok) {
+      if (!ok && leader) {
         abort_flag = 1;
         atomicExch(status, (int)WM_ERR_TIMEOUT);
         umma_commit(&drain_bar);   // every MMA issued above has finished

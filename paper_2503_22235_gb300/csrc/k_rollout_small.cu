@@ -28,7 +28,7 @@
 //               spin), then read their neighbours' K/V for the next block
 //
 // Roles (352 threads): warps 0-7 compute (attention, epilogues, LayerNorm),
-// warp 8 one thread issuing the tcgen05 MMAs, warp 9 one thread streaming the
+// warp 8 issuing the tcgen05 MMAs, warp 9 one thread streaming the
 // block's weights (12 pre-swizzled 32 KB chunks per block, one bulk copy each,
 // through a two-slot ring) and its biases and LayerNorm vectors (one bulk
 // copy into a two-slot buffer), warp 10 one thread issuing the K/V tensor
@@ -40,8 +40,11 @@
 // 21 %, QKV store 13 % of a 128-token patch's 67 k cycles; issue slots 41 %
 // busy), and one 4 x 24 x 48 latent in 128-token patches is 36 CTAs of 152
 // SMs: smaller patches put the idle SMs to work and shorten every phase but
-// the MMAs and the barrier. us per block: one latent 33.3 -> 16.9 (32 tokens,
-// 144 CTAs), two 33.3 -> 22.0 (64 tokens), three or four 33.6 as before (128 tokens).
+// the MMAs and the barrier. us per block: one latent 33.3 -> 16.5 (32 tokens,
+// 144 CTAs), two 33.3 -> 21.9 (64 tokens), three or four 33.6 -> 32.0 (128
+// tokens, by the MMA warp alone: its loop was inside one lane's branch, which
+// made the issue of every product a latency of its own; now the whole warp
+// walks it and one elected lane issues).
 // All patch sizes round alike, so the results do not depend on the choice.
 //
 // Every mbarrier wait and the latent barrier are bounded in time; on a
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int g = blockIdx.x / a.T, tile = blockIdx.x % a.T;
   const int nb = a.n6[g] * a.L6 + a.n1[g] * a.L1;   // blocks of this latent's rollout (>= 1)
   const int steps = NH * a.kd;                        // attention steps per block: (head of each group, key level)
@@ -519,25 +522,29 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
       }
     }
   } else if (warp == MMA_WARP) {
-    if (lane == 0) {
+    {
       // ------------------------------------------------------- MMA issuer
+      // (the whole warp walks the schedule, one elected lane issues)
+      const bool leader = elect_one();
       constexpr uint32_t idesc = idesc_bf16(128, 128);
       int slot = 0, par = 0, a_cnt = 0;
       bool ok = true;
       // one 128 x 128 x 128 product: A operand at a_addr, the next weight chunk of the ring
       auto gemm = [&](uint32_t col, uint32_t a_addr, bool acc_in) -> bool {
-        if (!mbar_wait(&w_full[slot], (uint32_t)par, &abort_flag)) return false;
+        if (!warp_wait(&w_full[slot], (uint32_t)par, &abort_flag)) return false;
         tc_fence_after();
         const uint32_t b_addr = sbase + OFF_W + slot * CHUNK;
+        if (leader) {
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const uint64_t ad = sw128_desc(a_addr + s * SLICE), bd = sw128_desc(b_addr + s * SLICE);
+          for (int s = 0; s < 2; ++s) {
+            const uint64_t ad = sw128_desc(a_addr + s * SLICE), bd = sw128_desc(b_addr + s * SLICE);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_bf16<false>(tmem + col, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc,
-                             (acc_in || s || k) ? 1u : 0u);
+            for (int k = 0; k < 4; ++k)
+              umma_bf16<false>(tmem + col, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc,
+                               (acc_in || s || k) ? 1u : 0u);
+          }
+          umma_commit(&w_empty[slot]);
         }
-        umma_commit(&w_empty[slot]);
         if (++slot == NSLOT) {
           slot = 0;
           par ^= 1;
@@ -545,7 +552,7 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         return true;
       };
       auto wait_a = [&]() -> bool {
-        const bool r = mbar_wait(&a_full, (uint32_t)(a_cnt++) & 1u, &abort_flag);
+        const bool r = warp_wait(&a_full, (uint32_t)(a_cnt++) & 1u, &abort_flag);
         tc_fence_after();
         return r;
       };
@@ -554,43 +561,45 @@ __global__ void __launch_bounds__(THREADS, 1) rollout_small_kernel(const __grid_
         if (!wait_a()) return false;
         for (int c = 0; c < 3; ++c)
           if (!gemm(T_ACC1 + 128 * c, A, false)) return false;
-        umma_commit(&mma_done);
+        if (leader) umma_commit(&mma_done);
         return true;
       };
       auto fc1 = [&](int j) -> bool {
         const int b = j & 1;
-        if (j >= 2 && !mbar_wait(&acc1_empty[b], 0u, &abort_flag)) return false;
+        if (j >= 2 && !warp_wait(&acc1_empty[b], 0u, &abort_flag)) return false;
         tc_fence_after();
         if (!gemm(T_ACC1 + 128 * b, A, false)) return false;
-        umma_commit(&acc1_full[b]);
+        if (leader) umma_commit(&acc1_full[b]);
         return true;
       };
       auto fc2 = [&](int j) -> bool {
         const int b = j & 1;
-        if (!mbar_wait(&h_full[b], (uint32_t)(j >> 1), &abort_flag)) return false;
+        if (!warp_wait(&h_full[b], (uint32_t)(j >> 1), &abort_flag)) return false;
         tc_fence_after();
         if (!gemm(T_ACC2, sbase + OFF_H + b * CHUNK, j > 0)) return false;
-        umma_commit(&h_empty[b]);
+        if (leader) umma_commit(&h_empty[b]);
         return true;
       };
       ok = qkv();
       for (int i = 0; i < nb && ok; ++i) {
         ok = wait_a() && gemm(T_PROJ, A, false);
         if (!ok) break;
-        umma_commit(&mma_done);
+        if (leader) umma_commit(&mma_done);
         ok = wait_a() && fc1(0) && fc1(1) && fc2(0) && fc1(2) && fc2(1) && fc1(3) && fc2(2) && fc2(3);
         if (!ok) break;
-        umma_commit(&mma_done);
+        if (leader) umma_commit(&mma_done);
         if (i + 1 < nb) ok = qkv();
       }
-      if (!ok) {
-        abort_flag = 1;
-        atomicExch(a.status, (int)WM_ERR_TIMEOUT);
+      if (leader) {
+        if (!ok) {
+          abort_flag = 1;
+          atomicExch(a.status, (int)WM_ERR_TIMEOUT);
+        }
+        // every MMA issued so far completes before TMEM and shared memory are released
+        umma_commit(&drain_bar);
+        volatile int never = 0;
+        mbar_wait(&drain_bar, 0u, &never);
       }
-      // every MMA issued so far completes before TMEM and shared memory are released
-      umma_commit(&drain_bar);
-      volatile int never = 0;
-      mbar_wait(&drain_bar, 0u, &never);
     }
   } else if (warp < 8) {
     // ------------------------------------------------------ compute warps
