@@ -800,7 +800,9 @@ struct RolloutTraffic {
 
  private:
   int peak() const { return std::max(1, *std::max_element(recent, recent + 8)); }
-} g_rollout_traffic;
+};
+// (never destroyed: a context may be given back while the process exits)
+RolloutTraffic& g_rollout_traffic = *new RolloutTraffic;
 
 // Tokens of a patch for G latents in one launch: fewer tokens a CTA shorten
 // every phase of a block, so a launch takes the smallest patches whose CTAs
