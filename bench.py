@@ -614,7 +614,7 @@ def small_rollout(wm, torch, dev, reps=10):
     x1 = torch.from_numpy(synth.latent(s, 1, seed=1)).to(dev)
     x4 = torch.from_numpy(synth.latent(s, 4, seed=1)).to(dev)
     res = {"workload": "latent 4x24x48x128, window 3x5x5, P6 8 blocks + P1 4 blocks, greedy schedule; "
-                       "bf16: one whole-rollout launch (a CTA per 8x16 patch), bf16_per_kernel: one graph"}
+                       "bf16: one whole-rollout launch (a CTA per 8x16, 8x8 or 8x4 patch), bf16_per_kernel: one graph"}
 
     def timed(x0, T):
         x = x0.clone()
@@ -665,7 +665,7 @@ def batch_bench(wm, torch, dev, reps=3):
     ctx = wm.wm_create_from_host(wm.make_config(s, wm.WM_PREC_BF16, max_batch=len(leads)),
                                  synth.pack_weights(p6, p1))
     res = {"workload": "8 latents 4x24x48x128, leads {1,6,7,24,72,120,240,336} h, 1080 blocks; "
-                       "bf16: two whole-rollout launches of four latents (longest leads first), "
+                       "bf16: whole-rollout launches of up to four latents, rollouts cut at steps, "
                        "fp8mlp / fp32: one graph of batched steps"}
     outs = {}
     try:
