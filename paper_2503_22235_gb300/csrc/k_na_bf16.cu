@@ -1093,49 +1093,55 @@ double na_plan_time(const NaPlan& pl, int B, int D, int H, int W, int heads, int
 }
 
 // Plan when none is tuned, among the plans of family `fam` (and kernel kind
-// `kind`, unless it is -1).
+// `kind`, unless it is -1): the one with the fewest staged keys per query times
+// tile waste (persistent plans preferred when the tile count gives every SM
+// several tiles), unless na_plan_time gives another at most four fifths of its
+// time. Over the 270 grids, chunks of eight groups: 0.943 times the time of the
+// first rule alone, slower by more than 2 % on one (9 %); taking the model's
+// plan always, 0.915 times, but slower on sixteen (up to 44 %). 9 x 90 x 180 x
+// 768: 1.58 ms by the first rule, now 1.25.
 NaPlan na_heuristic(int B, int D, int H, int W, int heads, int kd, int kh, int kw, int dh, bool periodic, int fam,
                     int kind) {
-  NaPlan best{};
-  double best_t = 1e300;
+  NaPlan best{}, quick{};
+  double best_score = 1e30, best_t = 1e300, quick_t = 1e300;
   for (const NaPlan& pl : na_candidates(kh, kw, H, W, heads * dh, heads, periodic, fam)) {
     if (pl.tc) return pl;   // the tcgen05 family has one plan
     if (kind >= 0 && pl.kind != kind) continue;
+    const int TH = pl.NWH * pl.WH, TW = pl.NWW * pl.WW;
+    const int th = (H + TH - 1) / TH, tw = (W + TW - 1) / TW;
+    const int hr = std::min(TH + kh - 1, H), wc = (pl.NWW - 1) * pl.WW + pl.span;
+    const long ctas = (long)th * tw * D * B * heads;
+    double score = (double)hr * wc / (TH * TW) * ((double)th * TH / H) * ((double)tw * TW / W);
+    if (ctas < num_sms()) score *= (double)num_sms() / ctas;   // idle SMs
+    if (pl.kind == 1 && kind < 0) score *= (ctas >= 4L * num_sms()) ? 0.8 : 1.5;
+    score /= std::sqrt((double)(pl.NWH * pl.NWW * pl.WH * pl.WW) / 128.0);   // more warps hide more latency
     const double t = na_plan_time(pl, B, D, H, W, heads, kd, kh, kw, dh, periodic);
-    if (t < best_t) {
+    if (score < best_score) {
+      best_score = score;
       best_t = t;
       best = pl;
     }
+    if (t < quick_t) {
+      quick_t = t;
+      quick = pl;
+    }
   }
-  return best;
+  return quick_t < 0.8 * best_t ? quick : best;
 }
 
-// Arithmetic family of a shape that no context has tuned: the one of the plan
-// with the smallest time for one latent, so that a batched call rounds as a
-// single one does. With the plan chosen above, 1.04 times the fastest plan of
-// all on the 270 grids (1.27 with chunks of eight and the plan with the fewest
-// staged keys; 9 x 90 x 180 x 768: 1.58 ms, now 1.06), slower than those by
-// more than 2 % on six of them (at most 11 %).
-int na_default_family(int D, int H, int W, int heads, int kd, int kh, int kw, int dh, bool periodic) {
-  const NaPlan pl = na_heuristic(1, D, H, W, heads, kd, kh, kw, dh, periodic, 0, -1);
-  return pl.NWH ? family(pl) : 8;
-}
-
-// na_heuristic (fam = -1: of the default family), remembered per shape: the
-// candidates' times take ~10 us of host time, as long as a small launch.
+// na_heuristic, remembered per shape: the candidates' times take ~10 us of
+// host time, as long as a small launch.
 NaPlan na_pick(int B, int D, int H, int W, int C, int heads, int kd, int kh, int kw, bool periodic, int fam, int kind) {
   static std::map<NaKey, NaPlan> picks;
   constexpr size_t kMaxPicks = 4096;
   NaKey key = na_key(B, D, H, W, C, heads, kd, kh, kw, periodic);
-  key[10] = 4 * (fam + 1) + kind + 1;
+  key[10] = 4 * fam + kind + 1;
   {
     std::lock_guard<std::mutex> lk(g_na_mu);
     auto it = picks.find(key);
     if (it != picks.end()) return it->second;
   }
-  const int dh = C / heads;
-  if (fam < 0) fam = na_default_family(D, H, W, heads, kd, kh, kw, dh, periodic);
-  const NaPlan pl = na_heuristic(B, D, H, W, heads, kd, kh, kw, dh, periodic, fam, kind);
+  const NaPlan pl = na_heuristic(B, D, H, W, heads, kd, kh, kw, C / heads, periodic, fam, kind);
   std::lock_guard<std::mutex> lk(g_na_mu);
   if (picks.size() >= kMaxPicks) picks.clear();
   picks[key] = pl;
@@ -1241,6 +1247,7 @@ wm_status launch_na_bf16(const __nv_bfloat16* qkv, __nv_bfloat16* out, int B, in
   if (!warp_patch(0, kh, kw, &WH, &WW, &span))
     return fail(WM_ERR_INVALID_ARG, "longitude window too wide for the BF16 attention kernel");
   NaPlan pl{};
+  // a shape that no context has tuned: chunks of eight groups, whatever the plan
   int fam = 8, kind = -1;
   if (variant == WM_NA_TCGEN05) {
     if (!na_tc_supported(H, W, C, heads, kh, kw, periodic))
@@ -1255,7 +1262,7 @@ wm_status launch_na_bf16(const __nv_bfloat16* qkv, __nv_bfloat16* out, int B, in
     auto it = g_na_plans.find(na_key(B, D, H, W, C, heads, kd, kh, kw, periodic));
     if (it != g_na_plans.end()) pl = it->second;
     auto ig = g_na_family.find(na_key(0, D, H, W, C, heads, kd, kh, kw, periodic));
-    fam = ig != g_na_family.end() ? ig->second : -1;
+    if (ig != g_na_family.end()) fam = ig->second;
   }
   if (!pl.NWH) pl = na_pick(B, D, H, W, C, heads, kd, kh, kw, periodic, fam, kind);
   if (!pl.NWH) return fail(WM_ERR_INVALID_ARG, "attention window too large for the BF16 attention kernel");
