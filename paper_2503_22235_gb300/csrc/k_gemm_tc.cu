@@ -171,6 +171,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, EPI), 1)
                         const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2, int M,
                         int N, int K, const EpiArgs e, int* __restrict__ status) {
   const float* __restrict__ bias = e.bias;
+  // a caller's bias may start at any float: 128-bit loads only where it is 16-byte aligned
+  const bool bias_vec = bias != nullptr && (reinterpret_cast<uintptr_t>(bias) & 15) == 0;
   const float alpha = e.alpha, out_scale = e.out_scale;
   constexpr bool kResLN = (EPI == EPI_RESID_LN);
   constexpr bool kLNF = (EPI == EPI_LNF_STORE || EPI == EPI_LNF_GELU);
@@ -451,8 +453,8 @@ __global__ void __launch_bounds__(gemm_threads(BN, EPI), 1)
               if constexpr (EPI == EPI_LNF_GELU) gelu_erf2(v[j], v[j + 1]);
             }
           }
-        } else if ((EPI == EPI_GELU || EPI == EPI_GELU_F8 || EPI == EPI_STORE) && bias && n + 32 <= N) {
-          // whole chunk with a bias: the same steps two columns per instruction
+        } else if ((EPI == EPI_GELU || EPI == EPI_GELU_F8 || EPI == EPI_STORE) && bias_vec && n + 32 <= N) {
+          // whole chunk with a bias in 128-bit loads: the same steps two columns per instruction
           const uint64_t alpha2 = pack_f2(alpha, alpha), oscale2 = pack_f2(out_scale, out_scale);
           const float4* b4 = reinterpret_cast<const float4*>(bias + n);
 #pragma unroll
