@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
     uint32_t phase = 0;
     bool ok = true;
     uint8_t* stg0 = smem + CF::OFF_OUT + (warp - CF::EPI) * 8192;   // 16-byte unit u of row r at u ^ (r & 7)
+    uint32_t staged = 0;   // chunks staged so far (all tiles; a ragged tile may skip its second)
     float acc[HC];
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
 #pragma unroll
@@ -467,16 +468,15 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
       if (!ok) break;
       const int row0 = (tile / num_n) * BM + quarter * 32, n0 = (tile % num_n) * BN + half * HC;
       if (row0 >= M) continue;
-      // 32 columns at a time through two staging tiles in turn
+      // 32 columns at a time, through the two staging tiles in turn
 #pragma unroll
       for (int c = 0; c < HC; c += 32) {
         const int n = n0 + c;
         if (n >= N) continue;
-        uint8_t* stg = stg0 + ((c >> 5) & 1) * 4096;
-        if (tma_out && lane == 0) {   // the copy that last used this tile has read it
-          if (HC > 32) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        }
+        uint8_t* stg = stg0 + (staged & 1u) * 4096;
+        ++staged;
+        // the copy that last used this staging tile, the one before the newest, has read it
+        if (tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         __syncwarp();
         bool any = false;
 #pragma unroll
