@@ -672,11 +672,15 @@ __global__ void __launch_bounds__(NaBlk<DH>::MAXT, 1)
         sc[j] = (cm >> j) & 1u ? f[0] * scale : -INFINITY;
         rmax = fmaxf(rmax, sc[j]);
       }
-      // The reference moves only when some score of the warp passes it by more
-      // than 8 (probabilities stay below e^8), so most rows rescale nothing.
-      if (__any_sync(0xffffffffu, rmax > m + 8.f)) {
-        const float mn = fmaxf(m, rmax);
-        const float a0 = expf(m - mn);   // 0 while m is the initial value: o and l are still zero
+      // The references of a block's queries move together, and only when some score
+      // of the block passes its query's by more than 8 (probabilities stay below
+      // e^8), so most rows rescale nothing. The vote is the block's alone: what
+      // shares its warp follows from the tile, which the batch size may change.
+      const uint32_t votes = __ballot_sync(0xffffffffu, rmax > m + 8.f);
+      if (votes != 0u) {
+        const bool moves = ((votes >> (threadIdx.x & 31 & ~(TPB - 1))) & ((1u << TPB) - 1u)) != 0u;
+        const float mn = moves ? fmaxf(m, rmax) : m;
+        const float a0 = moves ? expf(m - mn) : 1.f;   // 0 while m is the initial value: o and l are still zero
         l *= a0;
         m = mn;
         const float a1 = __shfl_xor_sync(0xffffffffu, a0, 2), a2 = __shfl_xor_sync(0xffffffffu, a0, 1),
