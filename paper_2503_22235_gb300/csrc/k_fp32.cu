@@ -496,8 +496,12 @@ __global__ void __launch_bounds__(256, 2) na_f32_tile_kernel(const float* __rest
 // window 5 x 7 x 7: 17.2 ms with one query per four threads (every K and V
 // value read for one query only), 4.4 ms here.
 // FP32 FMA and expf throughout. A masked key has probability zero; where its
-// V is not finite that makes the output NaN, and a NaN output is recomputed
-// over its own window alone.
+// V is not finite that makes the output NaN, and an output that is NaN although
+// the query's own scores are not is recomputed over its own window alone, by
+// the lanes of its block. 9 x 90 x 180 x 768: 4.4 ms with every token NaN or none,
+// 8.1 with one in 4001 and 16.5 with one in 50, whose neighbours are recomputed
+// (by one thread for each float4, whatever the scores: 380 ms with one in 4001,
+// seconds with more).
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -531,31 +535,60 @@ struct NaBlk {
   static constexpr int MAXT = DH == 48 ? 384 : 512;  // threads per CTA: 168 or 128 registers
 };
 
-// Four channels of one query's output over its own window, in two passes
-// (key0: K of the batch element and head; the channels' V lie C + ch floats on).
-__device__ __noinline__ void na_f32_query(const float* q, const float* key0, float* o, int ch, int H, int W, int C,
-                                          int dh, int ld0, int kd, int r0, int kh, int c0, int kw, float scale) {
-  float mx = -INFINITY, sum = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int pass = 0; pass < 2; ++pass)
-    for (int l = 0; l < kd; ++l)
-      for (int r = 0; r < kh; ++r)
-        for (int c = 0; c < kw; ++c) {
-          int lon = c0 + c;
-          while (lon < 0) lon += W;
-          while (lon >= W) lon -= W;
-          const float* key = key0 + (((long)(ld0 + l) * H + r0 + r) * W + lon) * 3 * C;
-          float sc = 0.f;
-          for (int e = 0; e < dh; ++e) sc = fmaf(q[e], key[e], sc);
-          sc *= scale;
-          if (pass == 0) {
-            mx = fmaxf(mx, sc);
-          } else {
-            const float p = expf(sc - mx);
-            sum += p;
-            for (int e = 0; e < 4; ++e) acc[e] = fmaf(p, key[C + ch + e], acc[e]);
-          }
+// The output of one query over its own window alone, by the TPB lanes `group` of
+// its block: each takes the block kernel's share of the channels of every key
+// (q, key0: the query's and the batch element's K of this head; V lies C floats
+// on), and a key's score is summed over the lanes. The softmax reference M and
+// 1 / sum are the block kernel's. Writes the float4 of the set `bits`.
+template <int DH, int KW>
+__device__ __noinline__ void na_f32_query(const float* q, const float* key0, float* o, uint32_t bits, uint32_t group,
+                                          int part, int H, int W, int C, int ld0, int kd, int r0, int kh, int c0,
+                                          float scale, float M, float inv) {
+  constexpr int TPB = NaBlk<DH>::TPB, NI = NaBlk<DH>::NI;
+  float4 qv[NI], acc[NI];
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    qv[i] = *reinterpret_cast<const float4*>(q + 4 * (i * TPB + part));
+    acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll 1
+  for (int l = 0; l < kd; ++l)
+#pragma unroll 1
+    for (int r = 0; r < kh; ++r) {
+      const float* row = key0 + ((long)(ld0 + l) * H + r0 + r) * W * 3 * C + 4 * part;
+      const float* key[KW];
+      float s[KW];
+#pragma unroll
+      for (int j = 0; j < KW; ++j) {
+        int lon = c0 + j;
+        while (lon < 0) lon += W;
+        while (lon >= W) lon -= W;
+        key[j] = row + (long)lon * 3 * C;
+        s[j] = 0.f;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const float4 k = *reinterpret_cast<const float4*>(key[j] + 4 * i * TPB);
+          s[j] = fmaf(qv[i].x, k.x, fmaf(qv[i].y, k.y, fmaf(qv[i].z, k.z, fmaf(qv[i].w, k.w, s[j]))));
         }
-  for (int e = 0; e < 4; ++e) o[ch + e] = acc[e] / sum;
+      }
+#pragma unroll
+      for (int j = 0; j < KW; ++j) {
+#pragma unroll
+        for (int d = 1; d < TPB; d *= 2) s[j] += __shfl_xor_sync(group, s[j], d);
+        const float p = expf(s[j] * scale - M) * inv;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const float4 v = *reinterpret_cast<const float4*>(key[j] + C + 4 * i * TPB);
+          acc[i].x = fmaf(p, v.x, acc[i].x);
+          acc[i].y = fmaf(p, v.y, acc[i].y);
+          acc[i].z = fmaf(p, v.z, acc[i].z);
+          acc[i].w = fmaf(p, v.w, acc[i].w);
+        }
+      }
+    }
+#pragma unroll
+  for (int i = 0; i < NI; ++i)
+    if ((bits >> i) & 1u) *reinterpret_cast<float4*>(o + 4 * (i * TPB + part)) = acc[i];
 }
 
 template <int DH, int KW>
@@ -741,12 +774,13 @@ __global__ void __launch_bounds__(NaBlk<DH>::MAXT, 1)
     f0[2 + k] = __shfl_xor_sync(0xffffffffu, f0[k], 1);
     f1[2 + k] = __shfl_xor_sync(0xffffffffu, f1[k], 1);
   }
-  uint32_t nan = 0u;   // float4 of a query at bit k NI + i
+  uint32_t bad = 0u;   // float4 i of query qi at bit qi NI + i
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int qi = own ^ k, hq = bh + (qi >> 1), wq = bw + (qi & 1);
     if (!ok || hq >= H || wq >= W) continue;
     float* orow = out + ((long)b * N + ((long)d * H + hq) * W + wq) * C + head * DH;
+    const bool sound = f0[k] == f0[k] && f1[k] == f1[k];   // else a score of the query's own is NaN: so is all of it
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       float y[4];
@@ -754,18 +788,28 @@ __global__ void __launch_bounds__(NaBlk<DH>::MAXT, 1)
       for (int e = 0; e < 4; ++e) {
         const float2 u = unpack2(o[k][2 * i + (e >> 1)]);
         y[e] = ((e & 1) ? u.y : u.x) * f0[k] + xs[(2 + 4 * NI * k + 4 * i + e) * nthr + ht] * f1[k];
-        if (y[e] != y[e]) nan |= 1u << (k * NI + i);
+        if (sound && y[e] != y[e]) bad |= 1u << (qi * NI + i);
       }
       *reinterpret_cast<float4*>(orow + 4 * (i * TPB + part)) = make_float4(y[0], y[1], y[2], y[3]);
     }
   }
+  if (__any_sync(0xffffffffu, bad != 0u)) {
+    const int lane0 = threadIdx.x & 31 & ~(TPB - 1);   // of the block's lanes
+    const uint32_t group = ((1u << TPB) - 1u) << lane0;
+    uint32_t need = 0u;   // queries of the block with such a float4 in any lane
+#pragma unroll
+    for (int qi = 0; qi < 4; ++qi)
+      need |= (__ballot_sync(0xffffffffu, ((bad >> (qi * NI)) & ((1u << NI) - 1u)) != 0u) & group) != 0u ? 1u << qi : 0u;
 #pragma unroll 1
-  for (; nan != 0u; nan &= nan - 1u) {
-    const int bit = __ffs(nan) - 1, qi = own ^ (bit / NI), hq = bh + (qi >> 1), wq = bw + (qi & 1);
-    const long tok = (long)b * N + ((long)d * H + hq) * W + wq;
-    na_f32_query(qkv + tok * C3 + head * DH, qkv + (long)b * N * C3 + C + head * DH, out + tok * C + head * DH,
-                 4 * ((bit % NI) * TPB + part), H, W, C, DH, ld0, kd, row_start(bh + (qi >> 1)) + hs0, kh,
-                 col_start(bw + (qi & 1)) + ws0, KW, scale);
+    for (; need != 0u; need &= need - 1u) {
+      const int qi = __ffs(need) - 1, hq = bh + (qi >> 1), wq = bw + (qi & 1);
+      const int owner = lane0 + ((qi >> 1) | ((qi & 1) << 1));
+      const float Mq = __shfl_sync(group, M, owner), iq = __shfl_sync(group, inv, owner);
+      const long tok = (long)b * N + ((long)d * H + hq) * W + wq;
+      na_f32_query<DH, KW>(qkv + tok * C3 + head * DH, qkv + (long)b * N * C3 + C + head * DH, out + tok * C + head * DH,
+                           (bad >> (qi * NI)) & ((1u << NI) - 1u), group, part, H, W, C, ld0, kd,
+                           row_start(bh + (qi >> 1)) + hs0, kh, col_start(bw + (qi & 1)) + ws0, scale, Mq, iq);
+    }
   }
 }
 
