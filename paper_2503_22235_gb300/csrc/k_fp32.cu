@@ -496,9 +496,10 @@ __global__ void __launch_bounds__(256, 2) na_f32_tile_kernel(const float* __rest
 // window 5 x 7 x 7: 17.2 ms with one query per four threads (every K and V
 // value read for one query only), 4.4 ms here.
 // FP32 FMA and expf throughout. A masked key has probability zero; where its
-// V is not finite that makes the output NaN, and an output that is NaN although
-// the query's own scores are not is recomputed over its own window alone, by
-// the lanes of its block. 9 x 90 x 180 x 768: 4.4 ms with every token NaN or none,
+// V is not finite that makes the output NaN, and a V above FLT_MAX / e^8 can
+// overflow before the division by the sum. An output that is not finite although
+// the query's own scores are is recomputed over its own window alone, with
+// probabilities already divided, by the lanes of its block. 9 x 90 x 180 x 768: 4.4 ms with every token NaN or none,
 // 8.1 with one in 4001 and 16.5 with one in 50, whose neighbours are recomputed
 // (by one thread for each float4, whatever the scores: 380 ms with one in 4001,
 // seconds with more).
@@ -788,7 +789,7 @@ __global__ void __launch_bounds__(NaBlk<DH>::MAXT, 1)
       for (int e = 0; e < 4; ++e) {
         const float2 u = unpack2(o[k][2 * i + (e >> 1)]);
         y[e] = ((e & 1) ? u.y : u.x) * f0[k] + xs[(2 + 4 * NI * k + 4 * i + e) * nthr + ht] * f1[k];
-        if (sound && y[e] != y[e]) bad |= 1u << (qi * NI + i);
+        if (sound && !(fabsf(y[e]) <= 3.402823466e38f)) bad |= 1u << (qi * NI + i);
       }
       *reinterpret_cast<float4*>(orow + 4 * (i * TPB + part)) = make_float4(y[0], y[1], y[2], y[3]);
     }
