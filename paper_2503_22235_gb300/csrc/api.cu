@@ -163,30 +163,36 @@ wm_status tune_block_gemms(wm_ctx* ctx, int batch);
 wm_status ensure_planes(wm_ctx* ctx) {
   if (ctx->planes_tried) return WM_OK;
   ctx->planes_tried = true;
-  const size_t C = ctx->cfg.C, kc = wm::f32_plane_k((int)C), k4 = wm::f32_plane_k((int)(4 * C));
-  const size_t per = 3 * (8 * C * kc + C * k4);   // Wqkv, Wo, W1 [8C rows of C], W2 [C rows of 4C]
+  const int C = ctx->cfg.C;
+  const size_t sizes[4] = {wm::f32_planes_size(3 * C, C), wm::f32_planes_size(C, C), wm::f32_planes_size(4 * C, C),
+                           wm::f32_planes_size(C, 4 * C)};   // Wqkv, Wo, W1, W2
+  const size_t per = sizes[0] + sizes[1] + sizes[2] + sizes[3];
   const size_t nb = ctx->blk[0].size() + ctx->blk[1].size();
   if (cudaMalloc(&ctx->d_wp, per * nb * 2) != cudaSuccess) {
     cudaGetLastError();
     ctx->d_wp = nullptr;
     return WM_OK;
   }
-  bf16* p = ctx->d_wp;
+  auto planes = [&](size_t block, int m) {
+    bf16* p = ctx->d_wp + block * per;
+    for (int i = 0; i < m; ++i) p += sizes[i];
+    return p;
+  };
+  size_t i = 0;
   for (auto& stack : ctx->blk)
     for (BlockW& w : stack) {
-      bf16* const q[4] = {p, p + 9 * C * kc, p + 12 * C * kc, p + 24 * C * kc};
-      WM_TRY(wm::launch_split_planes(w.wqkv, q[0], (int)(3 * C), (int)C, 0));
-      WM_TRY(wm::launch_split_planes(w.wo, q[1], (int)C, (int)C, 0));
-      WM_TRY(wm::launch_split_planes(w.w1, q[2], (int)(4 * C), (int)C, 0));
-      WM_TRY(wm::launch_split_planes(w.w2, q[3], (int)C, (int)(4 * C), 0));
-      p += per;
+      WM_TRY(wm::launch_split_planes(w.wqkv, planes(i, 0), 3 * C, C, 0));
+      WM_TRY(wm::launch_split_planes(w.wo, planes(i, 1), C, C, 0));
+      WM_TRY(wm::launch_split_planes(w.w1, planes(i, 2), 4 * C, C, 0));
+      WM_TRY(wm::launch_split_planes(w.w2, planes(i, 3), C, 4 * C, 0));
+      ++i;
     }
   WM_CUDA(cudaDeviceSynchronize());
-  p = ctx->d_wp;
+  i = 0;
   for (auto& stack : ctx->blk)
     for (BlockW& w : stack) {
-      w.p_qkv = p; w.p_o = p + 9 * C * kc; w.p_1 = p + 12 * C * kc; w.p_2 = p + 24 * C * kc;
-      p += per;
+      w.p_qkv = planes(i, 0); w.p_o = planes(i, 1); w.p_1 = planes(i, 2); w.p_2 = planes(i, 3);
+      ++i;
     }
   return WM_OK;
 }

@@ -44,10 +44,21 @@
 // tokens (C = 768) 13.41 -> 12.51 ms.
 //
 // NaN and infinity: a non-finite operand (or one that rounds up to infinity)
-// makes its second plane NaN, so every sum it enters comes out NaN. Operands
-// below 2^-110 lose their last planes (the tensor core takes bf16 subnormals
-// as zero). Outputs that are NaN, or not zero and below 2^-96, are recomputed
-// by the chain of FP32 FMAs, which gives what FP32 arithmetic gives.
+// makes its second plane NaN, so every sum it enters comes out NaN. Sums that
+// are not finite are recomputed by the chain of FP32 FMAs.
+// Small operands: the tensor core takes bf16 subnormals as zero, so an operand
+// may lose up to 2^-125 of itself (below 2^-110 its last planes, below 2^-126
+// all), and a product up to 2^-126. Where neither the row of A nor W has an
+// operand below 2^-48 (but zeros) nothing of that kind reaches 2^-25 of a
+// product. Else a sum of K products is off by at most K 2^-125 (max|w| + 3),
+// and K 2^-125 max|a| more where W has one: sums below 2^25 times that, zeros
+// included, are recomputed too. Ordinary sums are far above, whatever the
+// operands, so the epilogue compares first (with 2^30 for max|a|; a row that
+// passes it, which matters where W has small ones, is marked as it is split)
+// and looks for small operands in the row of A only where a sum is below. Where
+// it finds none (zero columns of W, zero rows), the splitting tests every
+// operand from then on, which costs 2 to 4 %. W's range comes from the
+// pre-pass, or from the splitting here.
 //
 // Every wait is bounded in time; on a timeout the CTA records WM_ERR_TIMEOUT,
 // its MMAs are drained, TMEM is freed and it returns.
@@ -114,26 +125,93 @@ __device__ __forceinline__ float* stage_at(uint8_t* stg, int r, int c) {
   return reinterpret_cast<float*>(stg + r * 128 + (((c >> 2) ^ (r & 7)) << 4) + (c & 3) * 4);
 }
 
-// A sum to be recomputed: NaN, or not zero and below 2^-96.
-__device__ __forceinline__ bool doubtful(float y) { return !(fabsf(y) >= 1.262177448e-29f) && y != 0.f; }
+constexpr float kSmall = 3.552713679e-15f, kLarge = 1073741824.f;   // 2^-48, 2^30
+constexpr float kMaxFloat = 3.402823466e38f;
 
-// Row r of a staged chunk (columns n ..): its doubtful sums by the plain chain
-// of FP32 FMAs.
-__device__ __forceinline__ void recompute_row(uint8_t* stg, int r, const float* a, const float* W, int n, int N,
-                                              int K) {
+// What operands span: the largest magnitude, and the smallest but zero (twice
+// its bits, less one). An infinity makes every sum it enters NaN: it counts for
+// no maximum.
+struct Range {
+  float hi = 0.f;
+  uint32_t lo = 0xffffffffu;
+  template <int N>
+  __device__ __forceinline__ void add(const float (&x)[N]) {
+    float m = 0.f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      m = fmaxf(m, fabsf(x[j]));
+      lo = __viaddmin_u32(__float_as_uint(x[j]) << 1, 0xffffffffu, lo);
+    }
+    if (m <= kMaxFloat) hi = fmaxf(hi, m);
+  }
+  // as one word: the magnitude, and the sign bit where one but zero is small
+  __device__ __forceinline__ uint32_t word() const {
+    return __float_as_uint(hi) | (lo < (__float_as_uint(kSmall) << 1) - 1u ? 0x80000000u : 0u);
+  }
+};
+__device__ __forceinline__ uint32_t range_merge(uint32_t a, uint32_t b) {
+  return max(a & 0x7fffffffu, b & 0x7fffffffu) | ((a | b) & 0x80000000u);
+}
+__device__ __forceinline__ uint32_t range_of_warp(uint32_t a) {
+  return __reduce_max_sync(0xffffffffu, a & 0x7fffffffu) | (__reduce_or_sync(0xffffffffu, a) & 0x80000000u);
+}
+
+// Sums below this are recomputed, by the ranges of A's row (its magnitude at most a_hi) and of W.
+__device__ __forceinline__ float doubt_below(float a_hi, uint32_t w, int K) {
+  if (w == 0u) return 0.f;   // W is zero
+  return (float)K * 3.155443621e-30f *   // 2^-98
+         (1.f + __uint_as_float(w & 0x7fffffffu) + ((w >> 31) != 0u ? a_hi : 0.f));
+}
+__device__ __forceinline__ bool doubtful(float y, float below) {
+  return !(fabsf(y) >= below) || !(fabsf(y) <= kMaxFloat);
+}
+
+// The threshold of this lane's row of A (from row0 on), for the rows in `look`;
+// w: W's range.
+__device__ __forceinline__ float look_at_rows(const float* A, int row0, int K, uint32_t look, uint32_t w) {
+  const int lane = threadIdx.x & 31;
+  float below = 0.f;
+  for (; look != 0u; look &= look - 1u) {
+    const int r = __ffs(look) - 1;
+    const float* a = A + (size_t)(row0 + r) * K;
+    Range ra;
+#pragma unroll 8
+    for (int k = lane; k < K; k += 32) {
+      const float x[1] = {__ldg(a + k)};
+      ra.add(x);
+    }
+    const uint32_t range = range_of_warp(ra.word());
+    if (lane == r && ((range | w) >> 31) != 0u) below = doubt_below(__uint_as_float(range & 0x7fffffffu), w, K);
+  }
+  return below;
+}
+
+// A staged chunk (rows row0 .., columns n ..) with sums that are not finite or
+// below `first`: each lane's row, in doubt below `below` or, in the rows `look`,
+// below what the row of A says, by the plain chain of FP32 FMAs. Returns
+// whether the look was in vain.
+__device__ __noinline__ bool recompute(uint8_t* stg, const float* A, const float* W, int row0, int M, int n, int N,
+                                       int K, uint32_t look, float below, uint32_t w) {
+  const int lane = threadIdx.x & 31;
+  const float looked = look_at_rows(A, row0, K, look, w);
+  const bool vain = look != 0u && (w >> 31) == 0u && !__any_sync(0xffffffffu, looked > 0.f);
+  if ((look >> lane) & 1u) below = looked;
+  if (row0 + lane >= M) return vain;
+  const float* a = A + (size_t)(row0 + lane) * K;
 #pragma unroll 1
   for (int e = 0; e < 32 && n + e < N; ++e) {
-    float* y = stage_at(stg, r, e);
-    if (!doubtful(*y)) continue;
-    const float* w = W + (size_t)(n + e) * K;
+    float* y = stage_at(stg, lane, e);
+    if (!doubtful(*y, below)) continue;
+    const float* wn = W + (size_t)(n + e) * K;
     float s = 0.f;
 #pragma unroll 1
     for (int k = 0; k < K; ++k) {
-      s = fmaf(a[k], w[k], s);
+      s = fmaf(a[k], wn[k], s);
       if (s != s) break;   // NaN stays NaN
     }
     *y = s;
   }
+  return vain;
 }
 
 // Tensor-core product with A from tensor memory (lane = row, two k a column).
@@ -153,13 +231,21 @@ __device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64
 template <int BN, bool TMA_A, bool PRE, bool VEC_W>
 __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
     gemm_f32_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
-                       const __grid_constant__ CUtensorMap tmC, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
-                       float* out, int M, int N, int K, int epi, int tma_out, int* __restrict__ status) {
+                       const __grid_constant__ CUtensorMap tmC, const float* __restrict__ A, const float* __restrict__ W,
+                       const float* __restrict__ bias,
+                       float* out, int M, int N, int K, int epi, int tma_out, const uint32_t* __restrict__ w_ranges,
+                       int num_ranges, int* __restrict__ status) {
   using CF = Cfg<BN, PRE>;
   constexpr int NACC = CF::NACC, CONV = CF::CONV;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t a_full[NA], a_empty[NA], planes_full[NST], planes_empty[NST];
   __shared__ __align__(8) uint64_t accf_bar[NACC], acce_bar[NACC], drain_bar;
+  // Whether a row of the tile held an operand above 2^30 (where W has small ones) or a small one (from the tile a_from
+  // of each splitting warp on, once a_watch asks for it), and the range of W by splitting warp; over all tiles so
+  // far: the splitting runs ahead, so they may hold more than the tile at hand, never less
+  __shared__ volatile uint32_t w_range[CONV];
+  __shared__ volatile uint8_t a_large[BM], a_small[BM];
+  __shared__ volatile int a_watch, a_from[CONV];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
 
@@ -185,8 +271,19 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
     }
     mbar_init(&drain_bar, 1);
     abort_flag = 0;
+    a_watch = 0;
+    for (int i = 0; i < CONV; ++i) {
+      w_range[i] = 0u;
+      a_from[i] = 0x7fffffff;
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (tid < BM) a_large[tid] = a_small[tid] = 0;
+  uint32_t rw = 0u;   // range of W: all of it, where the pre-pass took it, else what this warp has split or seen split
+  if constexpr (PRE) {
+    for (int i = lane; i < num_ranges; i += 32) rw = range_merge(rw, __ldg(w_ranges + i));
+    rw = range_of_warp(rw);
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_slot))
@@ -230,9 +327,15 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
     }
     int stage = 0, ia = 0;
     uint32_t phase = 0, aphase = 0;
-    bool ok = true;
+    bool ok = true, watch = (rw >> 31) != 0u;   // test the operands of A
+    if (watch && lane == 0) a_from[warp] = 0;
+    Range w_split;
     for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
       const int m = (tile / num_n) * BM + row;
+      if (PRE && !watch && __any_sync(0xffffffffu, a_watch != 0)) {
+        watch = true;
+        if (lane == 0) a_from[warp] = tile;
+      }
       for (int kb = 0; kb < nk; ++kb) {
         float x[KT];
         if constexpr (TMA_A) {
@@ -256,6 +359,12 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
 #pragma unroll
           for (int j = 0; j < KT; ++j) x[j] = m < M && k0 + j < K ? __ldg(p + j) : 0.f;
         }
+        if (PRE && watch) {
+          Range r;
+          r.add(x);
+          if (r.hi > kLarge) a_large[row] = 1;
+          if ((r.word() >> 31) != 0u) a_small[row] = 1;
+        }
         ok = __all_sync(0xffffffffu, mbar_wait(&planes_empty[stage], phase ^ 1u, &abort_flag));
         if (!ok) break;
         tc_fence_after();
@@ -277,12 +386,18 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
 #pragma unroll
           for (int i = 0; i < LDW; ++i) {
             float4 y = v[i];
+            const float y4[4] = {y.x, y.y, y.z, y.w};
+            w_split.add(y4);
             if (lt < num_tiles) v[i] = load_w(i, (lt % num_n) * BN, last ? 0 : (kb + 1) * BK);
             uint8_t* d = st + i * 32 * ROW;
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl)
               *reinterpret_cast<uint2*>(d + pl * CF::PLANE) =
                   pl < 2 ? make_uint2(split2(y.x, y.y), split2(y.z, y.w)) : make_uint2(bf16x2(y.x, y.y), bf16x2(y.z, y.w));
+          }
+          if (last) {
+            const uint32_t range = range_of_warp(w_split.word());
+            if (lane == 0) w_range[warp] = range;
           }
           fence_async_smem();
         }
@@ -468,6 +583,14 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
       if (!ok) break;
       const int row0 = (tile / num_n) * BM + quarter * 32, n0 = (tile % num_n) * BN + half * HC;
       if (row0 >= M) continue;
+      if constexpr (!PRE) {
+#pragma unroll
+        for (int i = 0; i < CONV; ++i) rw = range_merge(rw, w_range[i]);
+      }
+      // sums below `first` may need recomputing
+      const bool w_small = (rw >> 31) != 0u;
+      float first = doubt_below(kLarge, rw, K);
+      if (w_small && (!PRE || a_large[quarter * 32 + lane] != 0)) first = INFINITY;
       // 32 columns at a time, through the two staging tiles in turn
 #pragma unroll
       for (int c = 0; c < HC; c += 32) {
@@ -478,13 +601,32 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
         // the copy that last used this staging tile, the one before the newest, has read it
         if (tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         __syncwarp();
-        bool any = false;
+        // (a product with zero is NaN where the sum is not finite)
+        float z[4] = {}, least[2] = {INFINITY, INFINITY};
 #pragma unroll
-        for (int j = 0; j < 32; ++j) any = any || doubtful(acc[c + j]);
-        if (any && row0 + lane < M) {
+        for (int j = 0; j < 32; j += 4) {
+          fma_f2(z[0], z[1], acc[c + j], acc[c + j + 1], 0ull, pack_f2(z[0], z[1]));
+          fma_f2(z[2], z[3], acc[c + j + 2], acc[c + j + 3], 0ull, pack_f2(z[2], z[3]));
+          least[0] = fminf(fminf(least[0], fabsf(acc[c + j])), fabsf(acc[c + j + 1]));
+          least[1] = fminf(fminf(least[1], fabsf(acc[c + j + 2])), fabsf(acc[c + j + 3]));
+        }
+        if (n + 32 > N) {   // columns past N are zeros
+          least[0] = least[1] = INFINITY;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (n + j < N) least[0] = fminf(least[0], fabsf(acc[c + j]));
+        }
+        const bool low = row0 + lane < M && fminf(least[0], least[1]) < first;
+        if (__any_sync(0xffffffffu, low || (z[0] + z[1]) + (z[2] + z[3]) != 0.f)) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) *stage_at(stg, lane, j) = acc[c + j];
-          recompute_row(stg, lane, A + (size_t)(row0 + lane) * K, W, n, N, K);
+          uint32_t look = __ballot_sync(0xffffffffu, low);
+          float below = 0.f;
+          if (PRE && !w_small && tile >= a_from[quarter]) {   // known from the splitting
+            look = 0u;
+            if (a_small[quarter * 32 + lane] != 0) below = first;
+          }
+          if (recompute(stg, A, W, row0, M, n, N, K, look, below, rw)) a_watch = 1;
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc[c + j] = *stage_at(stg, lane, j);
         }
@@ -544,29 +686,51 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
   }
 }
 
-// W [N, K] as three planes [3][N][Kp] (Kp: K rounded up to a slab, zeros past K).
-__global__ void split_planes_kernel(const float* __restrict__ W, __nv_bfloat16* __restrict__ P, int N, int K, int Kp) {
+constexpr int kSplitThreads = 512, kMaxSplitBlocks = 256;
+int split_blocks(int N, int Kp) {
+  return (int)std::min<long>(((long)N * (Kp / 2) + kSplitThreads - 1) / kSplitThreads, kMaxSplitBlocks);
+}
+
+// W [N, K] as three planes [3][N][Kp] (Kp: K rounded up to a slab, zeros past
+// K), then each block's range of W.
+__global__ void __launch_bounds__(kSplitThreads)
+    split_planes_kernel(const float* __restrict__ W, __nv_bfloat16* __restrict__ P, int N, int K, int Kp) {
+  __shared__ uint32_t part[kSplitThreads / 32];
   const long total = (long)N * (Kp / 2), plane = (long)N * Kp;
+  Range r;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
     const int n = (int)(i / (Kp / 2)), k = 2 * (int)(i - (long)n * (Kp / 2));
     float x0 = k < K ? W[(size_t)n * K + k] : 0.f, x1 = k + 1 < K ? W[(size_t)n * K + k + 1] : 0.f;
+    const float x[2] = {x0, x1};
+    r.add(x);
     uint32_t* o = reinterpret_cast<uint32_t*>(P + (size_t)n * Kp + k);
     o[0] = split2(x0, x1);
     o[plane / 2] = split2(x0, x1);
     o[plane] = bf16x2(x0, x1);
   }
+  const uint32_t range = range_of_warp(r.word());
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = range;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const uint32_t all = range_of_warp(part[threadIdx.x & (kSplitThreads / 32 - 1)]);
+    if (threadIdx.x == 0) reinterpret_cast<uint32_t*>(P + 3 * plane)[blockIdx.x] = all;
+  }
 }
 
 template <int BN, bool TMA_A, bool PRE, bool VEC_W>
-wm_status launch_one(const CUtensorMap& tmA, const CUtensorMap& tmW, const float* A, const float* W, const float* bias,
-                     float* out, int M, int N, int K, int epi, cudaStream_t s) {
+wm_status launch_one(const CUtensorMap& tmA, const CUtensorMap& tmW, const float* A, const float* W,
+                     const __nv_bfloat16* planes, const float* bias, float* out, int M, int N, int K, int epi,
+                     cudaStream_t s) {
   const long tiles = (long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
   if (tiles > (1L << 30)) return fail(WM_ERR_INVALID_ARG, "too many FP32 GEMM tiles");
   const int grid = (int)std::min<long>(tiles, num_sms());
   CUtensorMap tmC{};
   const int tma_out = make_tmap_out(&tmC, out, (uint64_t)M, (uint64_t)N, true);   // false: unaligned rows
+  const int Kp = f32_plane_k(K);
+  const uint32_t* ranges = PRE ? reinterpret_cast<const uint32_t*>(planes + (size_t)3 * N * Kp) : nullptr;
   gemm_f32_tc_kernel<BN, TMA_A, PRE, VEC_W><<<grid, Cfg<BN, PRE>::THREADS, Cfg<BN, PRE>::SMEM, s>>>(
-      tmA, tmW, tmC, A, W, bias, out, M, N, K, epi, tma_out, device_status_word());
+      tmA, tmW, tmC, A, W, bias, out, M, N, K, epi, tma_out, ranges, PRE ? split_blocks(N, Kp) : 0,
+      device_status_word());
   WM_CUDA(cudaGetLastError());
   return WM_OK;
 }
@@ -579,11 +743,11 @@ wm_status launch_bn(const float* A, const float* W, const __nv_bfloat16* planes,
   if (planes && !make_tmap_planes(&tmW, planes, (uint64_t)N, (uint64_t)f32_plane_k(K), BN))
     return fail(WM_ERR_CUDA, "cuTensorMapEncodeTiled failed for the split weights");
   if (planes)
-    return tma_a ? launch_one<BN, true, true, false>(tmA, tmW, A, W, bias, out, M, N, K, epi, s)
-                 : launch_one<BN, false, true, false>(tmA, tmW, A, W, bias, out, M, N, K, epi, s);
+    return tma_a ? launch_one<BN, true, true, false>(tmA, tmW, A, W, planes, bias, out, M, N, K, epi, s)
+                 : launch_one<BN, false, true, false>(tmA, tmW, A, W, planes, bias, out, M, N, K, epi, s);
   const bool vec_w = K % 4 == 0 && (uintptr_t)W % 16 == 0;
-  if (tma_a && vec_w) return launch_one<BN, true, false, true>(tmA, tmW, A, W, bias, out, M, N, K, epi, s);
-  return launch_one<BN, false, false, false>(tmA, tmW, A, W, bias, out, M, N, K, epi, s);
+  if (tma_a && vec_w) return launch_one<BN, true, false, true>(tmA, tmW, A, W, planes, bias, out, M, N, K, epi, s);
+  return launch_one<BN, false, false, false>(tmA, tmW, A, W, planes, bias, out, M, N, K, epi, s);
 }
 
 template <int BN, bool TMA_A, bool PRE, bool VEC_W>
@@ -610,12 +774,13 @@ wm_status prepare_gemm_f32() {
 }
 
 int f32_plane_k(int K) { return (K + f32tc::BK - 1) / f32tc::BK * f32tc::BK; }
+size_t f32_planes_size(int N, int K) {
+  return (size_t)3 * N * f32_plane_k(K) + f32tc::kMaxSplitBlocks * sizeof(uint32_t) / sizeof(__nv_bfloat16);
+}
 
 wm_status launch_split_planes(const float* W, __nv_bfloat16* planes, int N, int K, cudaStream_t s) {
   const int Kp = f32_plane_k(K);
-  const long total = (long)N * (Kp / 2);
-  const int blocks = (int)std::min<long>((total + 255) / 256, (long)num_sms() * 8);
-  f32tc::split_planes_kernel<<<blocks, 256, 0, s>>>(W, planes, N, K, Kp);
+  f32tc::split_planes_kernel<<<f32tc::split_blocks(N, Kp), f32tc::kSplitThreads, 0, s>>>(W, planes, N, K, Kp);
   WM_CUDA(cudaGetLastError());
   return WM_OK;
 }
@@ -672,7 +837,7 @@ wm_status launch_linear_f32(const float* A, const float* W, const float* bias, f
   void* planes = nullptr;
   if (waves * nk > 16 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
     cudaMemPool_t pool = planes_pool();
-    const size_t bytes = (size_t)6 * N * f32_plane_k(K);
+    const size_t bytes = f32_planes_size(N, K) * sizeof(__nv_bfloat16);
     if (!pool || cudaMallocFromPoolAsync(&planes, bytes, pool, s) != cudaSuccess) {
       cudaGetLastError();
       planes = nullptr;

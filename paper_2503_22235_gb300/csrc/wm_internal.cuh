@@ -214,8 +214,10 @@ wm_status launch_row_stats(const float* x, __nv_bfloat16* xb, float* stats, int 
                            bool pdl = false);
 wm_status launch_layernorm_e4m3(const float* x, const float* g, const float* b, uint8_t* out, int M, int C,
                                 float eps, float inv_scale, cudaStream_t s, bool pdl = false);
-// planes: W split by launch_split_planes (3 N f32_plane_k(K) bf16), or NULL to split it inside the kernel.
+// planes: W split by launch_split_planes (f32_planes_size(N, K) bf16, a multiple of 16 bytes), or NULL to split it
+// inside the kernel.
 int f32_plane_k(int K);
+size_t f32_planes_size(int N, int K);
 wm_status launch_split_planes(const float* W, __nv_bfloat16* planes, int N, int K, cudaStream_t s);
 wm_status launch_gemm_f32(const float* A, const float* W, const __nv_bfloat16* planes, const float* bias, float* out,
                           int M, int N, int K, int epi, cudaStream_t s);
