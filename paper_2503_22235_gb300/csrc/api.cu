@@ -892,6 +892,13 @@ double rollout_small_time(const wm_config& c, const std::vector<RolloutPart>& pa
   return us;
 }
 
+wm_status alloc_rollout_done(wm_ctx* ctx) {
+  if (ctx->h_rs_done) return WM_OK;
+  WM_CUDA(cudaHostAlloc(&ctx->h_rs_done, sizeof(unsigned int), cudaHostAllocDefault));
+  *ctx->h_rs_done = 0;
+  return WM_OK;
+}
+
 // Once per context: every block's weights as 12 swizzled bf16 chunks and the
 // per-block table the kernel reads.
 wm_status prepare_rollout_small(wm_ctx* ctx) {
@@ -922,8 +929,7 @@ wm_status prepare_rollout_small(wm_ctx* ctx) {
   WM_CUDA(cudaMemcpy(ctx->d_rs_blk, tab.data(), tab.size() * sizeof(wm::RolloutBlock), cudaMemcpyHostToDevice));
   WM_CUDA(cudaMalloc(&ctx->d_rs_bar, wm::kRolloutSmallMaxLatents * sizeof(unsigned int)));
   WM_CUDA(cudaDeviceSynchronize());
-  WM_CUDA(cudaHostAlloc(&ctx->h_rs_done, sizeof(unsigned int), cudaHostAllocDefault));
-  *ctx->h_rs_done = 0;
+  WM_TRY(alloc_rollout_done(ctx));   // (there since the creation, where the context was made for this kernel)
   g_rollout_traffic.join(ctx);
   return WM_OK;
 }
@@ -1270,6 +1276,7 @@ wm_status wm_create_from_host(const wm_config* cfg, const float* weights, size_t
   wm_status st = upload_weights(ctx, weights, n_floats);
   if (st == WM_OK && cfg->rope) st = build_rope(ctx);
   if (st == WM_OK) st = ensure_workspace(ctx, ctx->cfg.max_batch);
+  if (st == WM_OK && rollout_small_shape(ctx->cfg)) st = alloc_rollout_done(ctx);
   if (st == WM_OK && cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     st = fail(WM_ERR_CUDA, "cudaStreamCreate failed");
   if (st == WM_OK && !wm::device_status_word()) st = fail(WM_ERR_OOM, "device status word allocation failed");
@@ -1557,7 +1564,8 @@ wm_status wm_autotune_report(char* buf, size_t len) {
 wm_status wm_ctx_reserve(wm_ctx* ctx, int batch) {
   if (!ctx || batch < 1) return fail(WM_ERR_INVALID_ARG, "bad reserve arguments");
   std::lock_guard<std::recursive_mutex> lk(ctx->mu);
-  return ensure_workspace(ctx, batch);
+  WM_TRY(ensure_workspace(ctx, batch));
+  return rollout_small_reserve(ctx, batch);
 }
 
 wm_status wm_timing_begin(wm_ctx* ctx, int max_launches) {
