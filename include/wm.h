@@ -384,6 +384,15 @@ wm_status wm_set_fused_mlp(int enable);
  * launch per GEMM / attention. WM_ERR_INVALID_ARG for another value. */
 wm_status wm_set_fused_rollout(int enable);
 
+/* Test hooks of the whole-rollout kernel. wm_rollout_patch_override forces its
+ * patches to 32, 64 or 128 tokens (0, the default: chosen by the library), in
+ * every launch made or captured afterwards; a launch whose patches do not fit
+ * on the device at once is then refused with WM_ERR_INVALID_ARG.
+ * wm_rollout_patch_tokens: the tokens of a patch in the context's last launch
+ * (HOST output; 0 before the first). (Library service.) */
+wm_status wm_rollout_patch_override(int tokens);
+wm_status wm_rollout_patch_tokens(wm_ctx* ctx, int* tokens);
+
 /* ------------------------------------------------------------------------
  * Encoder and decoder (Section 2.1 "Encoder-processor-decoder architecture";
  * Appendix A.1 variables, A.2 architecture). The paper gives the grid (0.25

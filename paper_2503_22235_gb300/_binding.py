@@ -86,6 +86,8 @@ _SIGS = {
     "wm_gemm_tile_override": (_c_int, [_c_int]),
     "wm_set_fused_mlp": (_c_int, [_c_int]),
     "wm_set_fused_rollout": (_c_int, [_c_int]),
+    "wm_rollout_patch_override": (_c_int, [_c_int]),
+    "wm_rollout_patch_tokens": (_c_int, [_vp, ctypes.POINTER(_c_int)]),
     "wm_codec_create": (_c_int, [ctypes.POINTER(wm_codec_config), _vp, _sz, ctypes.POINTER(_vp)]),
     "wm_codec_destroy": (_c_int, [_vp]),
     "wm_encode": (_c_int, [_vp, _vp, _vp, _vp, _vp, _vp]),
@@ -404,6 +406,18 @@ GEMM_TILES_TUNED, GEMM_TILES_128, GEMM_TILES_256, GEMM_TILES_PAIR, GEMM_TILES_64
 def wm_set_fused_rollout(enable) -> None:
     """1 (default): narrow-latent rollouts as one whole-rollout launch; 0: one launch per kernel."""
     _check(lib().wm_set_fused_rollout(int(enable)))
+
+
+def wm_rollout_patch_override(tokens) -> None:
+    """Test hook: force the whole-rollout kernel's patches to 32, 64 or 128 tokens; 0 restores the library's choice."""
+    _check(lib().wm_rollout_patch_override(int(tokens)))
+
+
+def wm_rollout_patch_tokens(ctx) -> int:
+    """Tokens of a patch in the context's last whole-rollout launch (0 before the first)."""
+    out = _c_int()
+    _check(lib().wm_rollout_patch_tokens(ctx, ctypes.byref(out)))
+    return out.value
 
 
 def wm_set_fused_mlp(enable) -> None:

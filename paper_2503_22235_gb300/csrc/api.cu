@@ -100,6 +100,7 @@ struct wm_ctx {
   unsigned int* h_rs_done = nullptr;      // pinned: the last launch that has ended
   unsigned int rs_seq = 0;                // the last launch made, and its stream (under g_rollout_traffic.mu)
   cudaStream_t rs_stream = nullptr;
+  int rs_tokens = 0;                      // of a patch in the last launch made
   std::recursive_mutex mu;
 };
 
@@ -332,6 +333,8 @@ std::atomic<int> g_mlp_fused{0};
 // 1: rollouts of eligible narrow latents run as one whole-rollout launch
 // (k_rollout_small.cu); 0: one launch per GEMM / attention as for any shape.
 std::atomic<int> g_fused_rollout{1};
+// Test hook (wm_rollout_patch_override): tokens of the whole-rollout kernel's patches, 0 = by rollout_small_tokens.
+std::atomic<int> g_rollout_patch{0};
 using GemmKey = std::array<long, 5>;   // rows (-1 for the residual epilogue), N, K, epilogue, e4m3
 std::mutex g_gemm_mu;
 std::map<GemmKey, GemmPick> g_gemm_picks;
@@ -818,6 +821,7 @@ RolloutTraffic& g_rollout_traffic = *new RolloutTraffic;
 // 128-token patches, 16.5 with 32; two 32, and 21.9 with 64. Four contexts
 // on four streams, one 64-block rollout each: 2213 us with 128, 4288 with 32.
 int rollout_small_tokens(const wm_config& c, int G, int streams) {
+  if (const int forced = g_rollout_patch.load()) return forced;
   int tokens = 128;
   for (int t : {64, 32})
     if (streams * G * c.D * (c.H / 8) * (c.W / (t / 8)) <= wm::rollout_small_capacity(t)) tokens = t;
@@ -990,6 +994,7 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   WM_CUDA(cudaMemsetAsync(ctx->d_rs_bar, 0, G * sizeof(unsigned int), s));
   wm::NvtxRange range("whole rollout (narrow latent)");
   WM_TRY(wm::launch_rollout_small(a, s));
+  ctx->rs_tokens = a.tokens;
   undo.ctx = nullptr;
   return WM_OK;
 }
@@ -1737,6 +1742,20 @@ wm_status wm_op_linear(const void* A, const void* W, const float* bias, void* ou
 wm_status wm_set_fused_rollout(int enable) {
   if (enable < 0 || enable > 1) return fail(WM_ERR_INVALID_ARG, "fused rollout switch must be 0 or 1");
   g_fused_rollout.store(enable);
+  return WM_OK;
+}
+
+wm_status wm_rollout_patch_override(int tokens) {
+  if (tokens != 0 && tokens != 32 && tokens != 64 && tokens != 128)
+    return fail(WM_ERR_INVALID_ARG, "rollout patches hold 32, 64 or 128 tokens (0: chosen by the library)");
+  g_rollout_patch.store(tokens);
+  return WM_OK;
+}
+
+wm_status wm_rollout_patch_tokens(wm_ctx* ctx, int* tokens) {
+  if (!ctx || !tokens) return fail(WM_ERR_INVALID_ARG, "NULL argument");
+  std::lock_guard<std::recursive_mutex> lk(ctx->mu);
+  *tokens = ctx->rs_tokens;
   return WM_OK;
 }
 
