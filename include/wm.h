@@ -389,7 +389,8 @@ wm_status wm_set_fused_rollout(int enable);
  * every launch made or captured afterwards; a launch whose patches do not fit
  * on the device at once is then refused with WM_ERR_INVALID_ARG.
  * wm_rollout_patch_tokens: the tokens of a patch in the context's last launch
- * (HOST output; 0 before the first). (Library service.) */
+ * (after wm_rollout_hourly, in its launches of one latent; HOST output; 0 before
+ * the first). (Library service.) */
 wm_status wm_rollout_patch_override(int tokens);
 wm_status wm_rollout_patch_tokens(wm_ctx* ctx, int* tokens);
 

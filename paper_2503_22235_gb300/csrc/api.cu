@@ -97,10 +97,11 @@ struct wm_ctx {
   float* d_rs_qkv = nullptr;              // its double-buffered bf16 q, k, v (capacity in floats)
   size_t rs_qkv_cap = 0;
   unsigned int* d_rs_bar = nullptr;       // one barrier counter per latent
-  unsigned int* h_rs_done = nullptr;      // pinned: the last launch that has ended
+  unsigned int* h_rs_done = nullptr;      // pinned: the last launch whose first patch is through
   unsigned int rs_seq = 0;                // the last launch made, and its stream (under g_rollout_traffic.mu)
   cudaStream_t rs_stream = nullptr;
   int rs_tokens = 0;                      // of a patch in the last launch made
+  int rs_streams = 0;                     // while a graph is captured: streams its launches share the device with
   std::recursive_mutex mu;
 };
 
@@ -820,6 +821,8 @@ RolloutTraffic& g_rollout_traffic = *new RolloutTraffic;
 // would take turns). us per block of 4 x 24 x 48: one latent 32 with
 // 128-token patches, 16.5 with 32; two 32, and 21.9 with 64. Four contexts
 // on four streams, one 64-block rollout each: 2213 us with 128, 4288 with 32.
+// (Streams whose launches wait for one another count as sharing: that costs
+// them the small patches, not results.)
 int rollout_small_tokens(const wm_config& c, int G, int streams) {
   if (const int forced = g_rollout_patch.load()) return forced;
   int tokens = 128;
@@ -967,8 +970,13 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   a.L6 = c.blocks_p6;
   a.L1 = c.blocks_p1;
   a.G = G;
-  const bool counted = cap == cudaStreamCaptureStatusNone;   // a captured launch runs later, any number of times
-  const int streams = counted ? g_rollout_traffic.enter(ctx, s, &a.seq) : g_rollout_traffic.seen();
+  // A captured launch runs later, any number of times: the library's own graphs
+  // are counted when they are launched (wm_rollout_hourly), a caller's graph keeps
+  // the patches of its capture.
+  const bool counted = cap == cudaStreamCaptureStatusNone;
+  const int streams = counted              ? g_rollout_traffic.enter(ctx, s, &a.seq)
+                      : ctx->rs_streams > 0 ? ctx->rs_streams
+                                            : g_rollout_traffic.seen();
   if (counted) a.done = ctx->h_rs_done;
   struct Undo {
     wm_ctx* ctx;
@@ -1618,7 +1626,18 @@ wm_status wm_rollout_hourly(wm_ctx* ctx, const float* x, int max_lead, float* ou
   cudaStream_t s = (cudaStream_t)stream;
   std::vector<uintptr_t> key = {3, (uintptr_t)x, (uintptr_t)out, (uintptr_t)max_lead, (uintptr_t)max_batch,
                                 (uintptr_t)ctx->cfg.precision};
-  return run_graph(ctx, key, s, [&](cudaStream_t st) -> wm_status {
+  // narrow latents: the graph's launches are sized for the streams in flight at
+  // this call, and the whole graph counts as one launch of this stream
+  const int G = rollout_small_group(ctx, std::min(max_batch, K + 1));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (G > 0) WM_CUDA(cudaStreamIsCapturing(s, &cap));
+  const bool counted = G > 0 && cap == cudaStreamCaptureStatusNone;
+  unsigned int seq = 0;
+  if (G > 0) {
+    ctx->rs_streams = counted ? g_rollout_traffic.enter(ctx, s, &seq) : g_rollout_traffic.seen();
+    for (int g = 1; g <= G; ++g) key.push_back((uintptr_t)rollout_small_tokens(ctx->cfg, g, ctx->rs_streams));
+  }
+  wm_status done = run_graph(ctx, key, s, [&](cudaStream_t st) -> wm_status {
     if (out != x) WM_CUDA(cudaMemcpyAsync(out, x, lat * 4, cudaMemcpyDeviceToDevice, st));
     // the six-hour anchors: out[6k] = P6(out[6(k-1)])
     for (int k = 1; k <= K; ++k) {
@@ -1645,6 +1664,11 @@ wm_status wm_rollout_hourly(wm_ctx* ctx, const float* x, int max_lead, float* ou
     }
     return WM_OK;
   });
+  if (G > 0) ctx->rs_tokens = rollout_small_tokens(ctx->cfg, 1, ctx->rs_streams);
+  ctx->rs_streams = 0;
+  if (counted && done == WM_OK) done = wm::launch_set_word(ctx->h_rs_done, seq, s);
+  if (counted && done != WM_OK) g_rollout_traffic.undo(ctx);
+  return done;
 }
 
 wm_status wm_rel_l2(const float* a, const float* b, size_t n, double* out, void* stream) {

@@ -77,6 +77,14 @@ wm_status prepare_kernels() {
 }
 
 // ---------------------------------------------------------------- casts ----
+__global__ void set_word_kernel(volatile unsigned int* word, unsigned int value) { *word = value; }
+
+wm_status launch_set_word(unsigned int* word, unsigned int value, cudaStream_t s) {
+  set_word_kernel<<<1, 1, 0, s>>>(word, value);
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
 __global__ void f32_to_bf16_kernel(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, size_t n) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = __float2bfloat16_rn(in[i]);

@@ -328,7 +328,7 @@ struct RolloutSmallArgs {
   const RolloutBlock* blk;   // device array: the six-hour blocks, then the one-hour blocks
   int L6, L1;                // blocks per processor
   int G, T;                  // latents; CTAs (patches) per latent
-  unsigned int* done;        // host word set to seq when the launch ends (nullptr: none)
+  unsigned int* done;        // host word set to seq when the launch's first patch is through (nullptr: none)
   unsigned int seq;
   int tokens;                // per patch: 128, 64 or 32 (8 latitudes x 16, 8 or 4 longitudes); results do not depend on it
   int D, H, W, kd, kh, kw;   // H % 8 == 0, W % 16 == 0, W >= 32, kh <= 5, kw <= 5, periodic longitude
@@ -340,6 +340,8 @@ struct RolloutSmallArgs {
   int* status;               // device status word
   float eps, scale_log2;     // LayerNorm epsilon; log2(e) / sqrt(32)
 };
+// A host word set in stream order.
+wm_status launch_set_word(unsigned int* word, unsigned int value, cudaStream_t s);
 // CTAs of patches of `tokens` tokens the device can hold at once for the rollout kernel (0 when unknown).
 int rollout_small_capacity(int tokens);
 wm_status launch_rollout_small(const RolloutSmallArgs& a, cudaStream_t s);
