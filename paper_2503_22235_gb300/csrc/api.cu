@@ -798,6 +798,11 @@ struct RolloutTraffic {
     *seq = ++ctx->rs_seq;
     return peak();
   }
+  // Contexts that may launch the kernel beside one another.
+  int holders() {
+    std::lock_guard<std::mutex> lk(mu);
+    return std::max(1, (int)users.size());
+  }
   int seen() {
     std::lock_guard<std::mutex> lk(mu);
     return peak();
@@ -971,12 +976,13 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   a.L1 = c.blocks_p1;
   a.G = G;
   // A captured launch runs later, any number of times: the library's own graphs
-  // are counted when they are launched (wm_rollout_hourly), a caller's graph keeps
-  // the patches of its capture.
+  // are counted when they are launched (wm_rollout_hourly); a caller's graph keeps
+  // the patches of its capture, small enough in number for every context there is
+  // to run beside it.
   const bool counted = cap == cudaStreamCaptureStatusNone;
   const int streams = counted              ? g_rollout_traffic.enter(ctx, s, &a.seq)
                       : ctx->rs_streams > 0 ? ctx->rs_streams
-                                            : g_rollout_traffic.seen();
+                                            : g_rollout_traffic.holders();
   if (counted) a.done = ctx->h_rs_done;
   struct Undo {
     wm_ctx* ctx;
@@ -1634,7 +1640,7 @@ wm_status wm_rollout_hourly(wm_ctx* ctx, const float* x, int max_lead, float* ou
   const bool counted = G > 0 && cap == cudaStreamCaptureStatusNone;
   unsigned int seq = 0;
   if (G > 0) {
-    ctx->rs_streams = counted ? g_rollout_traffic.enter(ctx, s, &seq) : g_rollout_traffic.seen();
+    ctx->rs_streams = counted ? g_rollout_traffic.enter(ctx, s, &seq) : g_rollout_traffic.holders();
     for (int g = 1; g <= G; ++g) key.push_back((uintptr_t)rollout_small_tokens(ctx->cfg, g, ctx->rs_streams));
   }
   wm_status done = run_graph(ctx, key, s, [&](cudaStream_t st) -> wm_status {

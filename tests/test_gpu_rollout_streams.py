@@ -44,3 +44,31 @@ def test_hourly_graphs_share_the_device():
     finally:
         for c in ctxs:
             wm.wm_destroy(c)
+
+
+def test_a_callers_graph_leaves_room_for_every_context():
+    """A captured step keeps its patches: they are sized for all contexts that there are."""
+    s = dataclasses.replace(synth.SMALL, blocks_p6=2, blocks_p1=1)
+    p6, p1 = synth.processor_weights(s, seed=5)
+    blob = synth.pack_weights(p6, p1)
+    ctxs = []
+    try:
+        for alive, tokens in ((1, 32), (2, 64), (4, 128)):
+            while len(ctxs) < alive:
+                ctxs.append(wm.wm_create_from_host(wm.make_config(s, wm.WM_PREC_BF16, 1), blob))
+                wm.wm_ctx_reserve(ctxs[-1], 1)
+            x = torch.from_numpy(synth.latent(s, 1, seed=1)).cuda()
+            ref = x.clone()
+            wm.wm_processor_step(ctxs[0], ref, wm.WM_P6)
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                wm.wm_processor_step(ctxs[0], x, wm.WM_P6)
+            assert wm.wm_rollout_patch_tokens(ctxs[0]) == tokens
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(x, ref)
+        wm.wm_device_status()
+    finally:
+        for c in ctxs:
+            wm.wm_destroy(c)
