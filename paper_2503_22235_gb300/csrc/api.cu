@@ -98,7 +98,7 @@ struct wm_ctx {
   size_t rs_qkv_cap = 0;
   unsigned int* d_rs_bar = nullptr;       // one barrier counter per latent
   unsigned int* h_rs_done = nullptr;      // pinned: the last launch whose first patch is through
-  unsigned int rs_seq = 0;                // the last launch made, and its stream (under g_rollout_traffic.mu)
+  unsigned int rs_seq = 0;                // the last launch made, and its stream (under its traffic's mu)
   cudaStream_t rs_stream = nullptr;
   int rs_tokens = 0;                      // of a patch in the last launch made
   int rs_streams = 0;                     // while a graph is captured: streams its launches share the device with
@@ -769,8 +769,8 @@ int rollout_small_group(const wm_ctx* ctx, int batch) {
   return std::min({batch, wm::kRolloutSmallMaxLatents, wm::rollout_small_capacity(128) / T});
 }
 
-// How many streams have whole-rollout launches in flight at once: the most
-// seen at any of the last eight launches.
+// How many streams have whole-rollout launches in flight at once on a device:
+// the most seen at any of its last eight launches.
 struct RolloutTraffic {
   std::mutex mu;
   std::vector<wm_ctx*> users;   // contexts that hold the kernel's weights
@@ -816,8 +816,11 @@ struct RolloutTraffic {
  private:
   int peak() const { return std::max(1, *std::max_element(recent, recent + 8)); }
 };
-// (never destroyed: a context may be given back while the process exits)
-RolloutTraffic& g_rollout_traffic = *new RolloutTraffic;
+// Of a context's device (never destroyed: a context may be given back while the process exits).
+RolloutTraffic& rollout_traffic(const wm_ctx* ctx) {
+  static RolloutTraffic* const devices = new RolloutTraffic[64];
+  return devices[ctx->device & 63];
+}
 
 // Tokens of a patch for G latents in one launch: fewer tokens a CTA shorten
 // every phase of a block, so a launch takes the smallest patches whose CTAs
@@ -942,7 +945,7 @@ wm_status prepare_rollout_small(wm_ctx* ctx) {
   WM_CUDA(cudaMalloc(&ctx->d_rs_bar, wm::kRolloutSmallMaxLatents * sizeof(unsigned int)));
   WM_CUDA(cudaDeviceSynchronize());
   WM_TRY(alloc_rollout_done(ctx));   // (there since the creation, where the context was made for this kernel)
-  g_rollout_traffic.join(ctx);
+  rollout_traffic(ctx).join(ctx);
   return WM_OK;
 }
 
@@ -980,13 +983,13 @@ wm_status rollout_small(wm_ctx* ctx, float* const* x, const int* n6, const int* 
   // the patches of its capture, small enough in number for every context there is
   // to run beside it.
   const bool counted = cap == cudaStreamCaptureStatusNone;
-  const int streams = counted              ? g_rollout_traffic.enter(ctx, s, &a.seq)
+  const int streams = counted              ? rollout_traffic(ctx).enter(ctx, s, &a.seq)
                       : ctx->rs_streams > 0 ? ctx->rs_streams
-                                            : g_rollout_traffic.holders();
+                                            : rollout_traffic(ctx).holders();
   if (counted) a.done = ctx->h_rs_done;
   struct Undo {
     wm_ctx* ctx;
-    ~Undo() { if (ctx) g_rollout_traffic.undo(ctx); }
+    ~Undo() { if (ctx) rollout_traffic(ctx).undo(ctx); }
   } undo{counted ? ctx : nullptr};
   a.tokens = rollout_small_tokens(c, G, streams);
   a.T = c.D * (c.H / 8) * (c.W / (a.tokens / 8));
@@ -1347,7 +1350,7 @@ wm_status wm_destroy(wm_ctx* ctx) {
   cudaFree(ctx->d_rs_blk);
   cudaFree(ctx->d_rs_qkv);
   cudaFree(ctx->d_rs_bar);
-  g_rollout_traffic.leave(ctx);
+  rollout_traffic(ctx).leave(ctx);
   cudaFreeHost(ctx->h_rs_done);
   cudaFree(ctx->d_stage);
   cudaFree(ctx->d_io);
@@ -1518,7 +1521,7 @@ wm_status wm_rollout_batch(wm_ctx* ctx, float* const* latents, const int* lead_h
     // narrow latent: launches of up to G latents with their own schedules,
     // read and written in place (no gather)
     const wm_config& c = ctx->cfg;
-    const int streams = g_rollout_traffic.seen();
+    const int streams = rollout_traffic(ctx).seen();
     std::vector<RolloutPart> parts = rollout_small_plan(c, G, n6, n1, false, streams);
     std::vector<RolloutPart> cut = rollout_small_plan(c, G, n6, n1, true, streams);
     if (rollout_small_time(c, cut, streams) < rollout_small_time(c, parts, streams)) parts.swap(cut);
@@ -1640,7 +1643,7 @@ wm_status wm_rollout_hourly(wm_ctx* ctx, const float* x, int max_lead, float* ou
   const bool counted = G > 0 && cap == cudaStreamCaptureStatusNone;
   unsigned int seq = 0;
   if (G > 0) {
-    ctx->rs_streams = counted ? g_rollout_traffic.enter(ctx, s, &seq) : g_rollout_traffic.holders();
+    ctx->rs_streams = counted ? rollout_traffic(ctx).enter(ctx, s, &seq) : rollout_traffic(ctx).holders();
     for (int g = 1; g <= G; ++g) key.push_back((uintptr_t)rollout_small_tokens(ctx->cfg, g, ctx->rs_streams));
   }
   wm_status done = run_graph(ctx, key, s, [&](cudaStream_t st) -> wm_status {
@@ -1673,7 +1676,7 @@ wm_status wm_rollout_hourly(wm_ctx* ctx, const float* x, int max_lead, float* ou
   if (G > 0) ctx->rs_tokens = rollout_small_tokens(ctx->cfg, 1, ctx->rs_streams);
   ctx->rs_streams = 0;
   if (counted && done == WM_OK) done = wm::launch_set_word(ctx->h_rs_done, seq, s);
-  if (counted && done != WM_OK) g_rollout_traffic.undo(ctx);
+  if (counted && done != WM_OK) rollout_traffic(ctx).undo(ctx);
   return done;
 }
 

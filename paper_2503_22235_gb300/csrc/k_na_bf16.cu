@@ -1135,6 +1135,7 @@ NaPlan na_pick(int B, int D, int H, int W, int C, int heads, int kd, int kh, int
   static std::map<NaKey, NaPlan> picks;
   constexpr size_t kMaxPicks = 4096;
   NaKey key = na_key(B, D, H, W, C, heads, kd, kh, kw, periodic);
+  key[9] += 2 * num_sms();   // the rule looks at nothing else of the device
   key[10] = 4 * fam + kind + 1;
   {
     std::lock_guard<std::mutex> lk(g_na_mu);

@@ -990,10 +990,11 @@ namespace rs {
 
 template <int TP>
 int capacity() {
-  static std::atomic<int> cap{-1};
-  if (cap >= 0) return cap;
+  static std::atomic<int> caps[64];   // by device, plus one
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::atomic<int>& cap = caps[dev & 63];
+  if (cap > 0) return cap - 1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   if (cudaFuncSetAttribute(rollout_small_kernel<TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<TP>::SMEM) !=
       cudaSuccess)
@@ -1001,8 +1002,8 @@ int capacity() {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, rollout_small_kernel<TP>, THREADS, Cfg<TP>::SMEM) !=
       cudaSuccess)
     return 0;
-  cap = per * sms;
-  return cap;
+  cap = per * sms + 1;
+  return per * sms;
 }
 
 template <int TP>
