@@ -8,11 +8,12 @@ and FP32 residual stream; seeded synthetic latent ~ N(0,1) and Xavier-uniform
 random weights (the paper's trained weights and ERA-5 data are not available).
 Metric: forecasts/s (six-hour latent forecasts of the full-size latent).
 
-Also reported on the same line: the plain FP32 GPU path on the same step and
-its BF16-vs-FP32 error, an end-to-end number through the host-buffer C-ABI
-call, the dominant kernel's roofline fraction from per-launch CUDA events, the
-14-day rollout on the 4 x 24 x 48 x 128 latent, and the FP64 CPU oracle timed
-on a bounded sample.
+Also measured: the plain FP32 GPU path on the same step and its BF16-vs-FP32
+error, an end-to-end number through the host-buffer C-ABI call, the dominant
+kernel's roofline fraction from per-launch CUDA events, the 14-day rollout on
+the 4 x 24 x 48 x 128 latent, serving, and the FP64 CPU oracle timed on a
+bounded sample. One JSON line on stdout holds the result and the main figure of
+each of these; the whole record, with every list, is a JSON line on stderr.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 Multi-GPU (replicas, weak scaling): torchrun --nproc-per-node N bench.py --gpus N ...
@@ -537,9 +538,48 @@ def run_ours(args):
                 "forecasts_per_s": 1.0 / info, "threads": ORACLE_ROLLOUT_THREADS}
             out["rollout_error_vs_oracle"] = rollout_error_curve(wm, torch, dev, steps)
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        print(json.dumps(out), file=sys.stderr, flush=True)   # the whole record
+        print(json.dumps(result_line(out)), flush=True)
     if ws > 1:
         torch.distributed.destroy_process_group()
+
+
+# One figure of each further section for the result line; the sections are in the record.
+SECTION_FIGURES = {
+    "fp32_plain": ("value", "bf16_vs_fp32_rel_l2"),
+    "fp8mlp": ("value", "fp8mlp_vs_fp32_rel_l2"),
+    "fields_14d_full": ("encode_ms", "decode_ms", "forecasts_per_s"),
+    "rollout_14d_small": ("bf16_T336_forecasts_per_s", "bf16_batch4_T336_forecasts_per_s"),
+    "batch_uneven_small": ("bf16_forecasts_per_s",),
+    "hourly_small_14d": ("forecast_sets_per_s",),
+    "ensemble_small_14d": ("member_forecasts_per_s",),
+    "ensemble_full_6h": ("member_forecasts_per_s",),
+    "serve": ("bf16_p50_ms", "bf16_p99_ms", "bf16_saturated_forecasts_per_s"),
+}
+
+
+def result_line(out):
+    """The one line on stdout: every key that says what was measured and how, and one or two figures of the further
+    sections. Lists by step and by plan make the whole record some 25 KB, more than readers of a log's tail keep."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks")
+    line = {k: out[k] for k in keys if k in out}
+    if "e2e" in out:
+        line["e2e"] = {k: v for k, v in out["e2e"].items() if k not in ("clocks", "single_call")}
+    line["roofline"] = {k: v for k, v in out["roofline"].items()
+                        if k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "peak_source",
+                                 "kernels_ms_per_step")}
+    for name, figures in SECTION_FIGURES.items():
+        if name in out:
+            line[name] = {k: out[name][k] for k in figures if k in out[name]}
+    curve = out.get("rollout_error_vs_oracle")
+    if curve:
+        line["rollout_error_vs_oracle"] = {prec: {k: r[k] for k in ("final_336h", "final_337h", "max")}
+                                           for prec, r in curve.items() if isinstance(r, dict)}
+    cpu = out.get("cpu_baseline")
+    if cpu:
+        line["cpu_baseline"] = {k: cpu[k] for k in ("value", "unit", "cores", "kind") if k in cpu}
+    return line
 
 
 def attn_halo(report, shape):
