@@ -41,7 +41,8 @@
 // N = 512, K = 128 with GELU: 22.5 and 15.2 us. The loop that issues the MMAs
 // inside one lane's branch left the tensor pipe idle between slabs; walked by
 // the whole warp, one elected lane issuing: 149 -> 136 us, a block of 145,800
-// tokens (C = 768) 13.41 -> 12.51 ms.
+// tokens (C = 768) 13.41 -> 12.51 ms, both the same within 1 % with the look for
+// small operands below.
 //
 // NaN and infinity: a non-finite operand (or one that rounds up to infinity)
 // makes its second plane NaN, so every sum it enters comes out NaN. Sums that
@@ -57,13 +58,15 @@
 // passes it, which matters where W has small ones, is marked as it is split)
 // and looks for small operands in the row of A only where a sum is below. Where
 // it finds none (zero columns of W, zero rows), the splitting tests every
-// operand from then on, which costs 2 to 4 %. W's range comes from the
-// pre-pass, or from the splitting here.
+// operand from then on, which costs 2 to 4 % (72,900 x 768 x 768: 350 us, 415
+// with a zero column, 610 with a look at every such row). W's range comes from
+// the pre-pass, or from the splitting here.
 //
 // Every wait is bounded in time; on a timeout the CTA records WM_ERR_TIMEOUT,
 // its MMAs are drained, TMEM is freed and it returns.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "tc_gemm.cuh"
 
@@ -336,80 +339,86 @@ __global__ void __launch_bounds__(Cfg<BN, PRE>::THREADS, 1)
         watch = true;
         if (lane == 0) a_from[warp] = tile;
       }
-      for (int kb = 0; kb < nk; ++kb) {
-        float x[KT];
-        if constexpr (TMA_A) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&a_full[ia], aphase, &abort_flag));
-          if (!ok) break;
-          const uint8_t* src = smem + CF::OFF_A + ia * A_BYTES + row * 128;
+      // (two loops: a branch in the one held up every slab, 3 % of a projection of 145,800 x 768 x 768)
+      auto slabs = [&](auto tag) {
+        constexpr bool kWatch = PRE && decltype(tag)::value;
+        for (int kb = 0; kb < nk; ++kb) {
+          float x[KT];
+          if constexpr (TMA_A) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&a_full[ia], aphase, &abort_flag));
+            if (!ok) return;
+            const uint8_t* src = smem + CF::OFF_A + ia * A_BYTES + row * 128;
 #pragma unroll
-          for (int j = 0; j < KT / 4; ++j) {
-            const float4 t = *reinterpret_cast<const float4*>(src + (((KT / 4 * hk + j) ^ (row & 7)) << 4));
-            x[4 * j] = t.x; x[4 * j + 1] = t.y; x[4 * j + 2] = t.z; x[4 * j + 3] = t.w;
+            for (int j = 0; j < KT / 4; ++j) {
+              const float4 t = *reinterpret_cast<const float4*>(src + (((KT / 4 * hk + j) ^ (row & 7)) << 4));
+              x[4 * j] = t.x; x[4 * j + 1] = t.y; x[4 * j + 2] = t.z; x[4 * j + 3] = t.w;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&a_empty[ia]);
+            if (++ia == NA) {
+              ia = 0;
+              aphase ^= 1u;
+            }
+          } else {
+            const int k0 = kb * BK + KT * hk;
+            const float* p = A + (size_t)m * K + k0;
+#pragma unroll
+            for (int j = 0; j < KT; ++j) x[j] = m < M && k0 + j < K ? __ldg(p + j) : 0.f;
           }
+          if constexpr (kWatch) {
+            Range r;
+            r.add(x);
+            if (r.hi > kLarge) a_large[row] = 1;
+            if ((r.word() >> 31) != 0u) a_small[row] = 1;
+          }
+          ok = __all_sync(0xffffffffu, mbar_wait(&planes_empty[stage], phase ^ 1u, &abort_flag));
+          if (!ok) return;
+          tc_fence_after();
+#pragma unroll
+          for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+            for (int h = 0; h < KT; h += 16) {
+              uint32_t w[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                w[j] = pl < 2 ? split2(x[h + 2 * j], x[h + 2 * j + 1]) : bf16x2(x[h + 2 * j], x[h + 2 * j + 1]);
+              tmem_st8(ta + (uint32_t)(stage * A_COLS + pl * (BK / 2) + h / 2), w);
+            }
+          if constexpr (!PRE) {
+            // the slab after this one
+            const bool last = kb + 1 == nk;
+            const int lt = last ? tile + (int)gridDim.x : tile;
+            uint8_t* st = smem + stage * CF::STAGE + soff;
+#pragma unroll
+            for (int i = 0; i < LDW; ++i) {
+              float4 y = v[i];
+              const float y4[4] = {y.x, y.y, y.z, y.w};
+              w_split.add(y4);
+              if (lt < num_tiles) v[i] = load_w(i, (lt % num_n) * BN, last ? 0 : (kb + 1) * BK);
+              uint8_t* d = st + i * 32 * ROW;
+#pragma unroll
+              for (int pl = 0; pl < 3; ++pl)
+                *reinterpret_cast<uint2*>(d + pl * CF::PLANE) = pl < 2 ? make_uint2(split2(y.x, y.y), split2(y.z, y.w))
+                                                                       : make_uint2(bf16x2(y.x, y.y), bf16x2(y.z, y.w));
+            }
+            if (last) {
+              const uint32_t range = range_of_warp(w_split.word());
+              if (lane == 0) w_range[warp] = range;
+            }
+            fence_async_smem();
+          }
+          tmem_wait_st();
+          tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&a_empty[ia]);
-          if (++ia == NA) {
-            ia = 0;
-            aphase ^= 1u;
+          if (lane == 0) mbar_arrive(&planes_full[stage]);
+          if (++stage == NST) {
+            stage = 0;
+            phase ^= 1u;
           }
-        } else {
-          const int k0 = kb * BK + KT * hk;
-          const float* p = A + (size_t)m * K + k0;
-#pragma unroll
-          for (int j = 0; j < KT; ++j) x[j] = m < M && k0 + j < K ? __ldg(p + j) : 0.f;
         }
-        if (PRE && watch) {
-          Range r;
-          r.add(x);
-          if (r.hi > kLarge) a_large[row] = 1;
-          if ((r.word() >> 31) != 0u) a_small[row] = 1;
-        }
-        ok = __all_sync(0xffffffffu, mbar_wait(&planes_empty[stage], phase ^ 1u, &abort_flag));
-        if (!ok) break;
-        tc_fence_after();
-#pragma unroll
-        for (int pl = 0; pl < 3; ++pl)
-#pragma unroll
-          for (int h = 0; h < KT; h += 16) {
-            uint32_t w[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              w[j] = pl < 2 ? split2(x[h + 2 * j], x[h + 2 * j + 1]) : bf16x2(x[h + 2 * j], x[h + 2 * j + 1]);
-            tmem_st8(ta + (uint32_t)(stage * A_COLS + pl * (BK / 2) + h / 2), w);
-          }
-        if constexpr (!PRE) {
-          // the slab after this one
-          const bool last = kb + 1 == nk;
-          const int lt = last ? tile + (int)gridDim.x : tile;
-          uint8_t* st = smem + stage * CF::STAGE + soff;
-#pragma unroll
-          for (int i = 0; i < LDW; ++i) {
-            float4 y = v[i];
-            const float y4[4] = {y.x, y.y, y.z, y.w};
-            w_split.add(y4);
-            if (lt < num_tiles) v[i] = load_w(i, (lt % num_n) * BN, last ? 0 : (kb + 1) * BK);
-            uint8_t* d = st + i * 32 * ROW;
-#pragma unroll
-            for (int pl = 0; pl < 3; ++pl)
-              *reinterpret_cast<uint2*>(d + pl * CF::PLANE) =
-                  pl < 2 ? make_uint2(split2(y.x, y.y), split2(y.z, y.w)) : make_uint2(bf16x2(y.x, y.y), bf16x2(y.z, y.w));
-          }
-          if (last) {
-            const uint32_t range = range_of_warp(w_split.word());
-            if (lane == 0) w_range[warp] = range;
-          }
-          fence_async_smem();
-        }
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&planes_full[stage]);
-        if (++stage == NST) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
+      };
+      if (PRE && watch) slabs(std::true_type{});
+      else slabs(std::false_type{});
     }
     if (!ok) {
       abort_flag = 1;
