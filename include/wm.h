@@ -115,12 +115,16 @@ wm_status wm_set_precision(wm_ctx* ctx, int precision);
 
 /* Sizes for `batch` latents at the context's current precision: floats per
  * latent (D*H*W*C) and bytes of the workspace the compute calls need (HOST
- * outputs, both required; WM_ERR_INVALID_ARG otherwise). (Library service.) */
+ * outputs, both required; WM_ERR_INVALID_ARG otherwise). Weights are not
+ * counted, nor is the split copy of them that a context keeps from its first
+ * FP32 use (creation, reserve or call) on: 6 bytes a matrix element, or none
+ * where there is no memory for it (slower, same results). (Library service.) */
 wm_status wm_ctx_sizes(wm_ctx* ctx, int batch, size_t* latent_floats, size_t* workspace_bytes);
 
 /* Allocate the workspace for `batch` latents now (at the current precision),
- * so that later calls, and graph captures, allocate nothing. WM_ERR_OOM if
- * it does not fit. (Library service.) */
+ * and what the whole-rollout kernel needs where it takes them, so that later
+ * calls, and graph captures, allocate nothing. WM_ERR_OOM if it does not fit.
+ * (Library service.) */
 wm_status wm_ctx_reserve(wm_ctx* ctx, int batch);
 
 /* The tile plans the autotuner chose so far in this process (text, one line
@@ -265,7 +269,7 @@ const char* wm_last_error(void);
  * lead time. They are admitted into device-resident latent slots in arrival
  * order while slots are free; the number of slots is set by the HBM budget:
  *   slots = (hbm_budget_bytes - workspace(max_batch) - max_batch latents of
- *            staging) / latent bytes.
+ *            staging) / latent bytes   (weights are not part of the budget).
  * Each tick, every admitted request with steps left takes one processor step
  * (greedy schedule, six-hour steps first); the requests due for the same
  * processor run as batched steps of at most max_batch latents; requests that
@@ -315,12 +319,17 @@ wm_status wm_op_layernorm(const float* x, const float* gamma, const float* beta,
                           int M, int C, float eps, void* stream);
 
 /* Linear layer D = A W^T + bias on A [M, K], W [N, K] (row major, K contiguous).
- * precision WM_PREC_FP32: A, W float32 (products exact to 2^-25, FP32 accumulate);
+ * precision WM_PREC_FP32: A, W float32 (products exact to 2^-25, FP32 accumulate;
+ * results that small operands or an overflow on the way would spoil are
+ * recomputed as a chain of FP32 FMAs). Larger calls split W beforehand in
+ * stream-ordered device memory, 6 bytes an element of W, of a pool that keeps at
+ * most 64 MB a device for later calls; inside a capture, or without memory,
+ * nothing is allocated;
  * precision WM_PREC_BF16: A, W bfloat16 (tcgen05, FP32 accumulate), K % 8 == 0.
  * epilogue 0: out = D (out float32 for FP32, bfloat16 for BF16)
  * epilogue 1: out = GELU(D) (same out types)
  * epilogue 2: out (float32 [M, N]) += D   (residual add)
- * epilogue 3: out (float32) = D. bias may be NULL. */
+ * epilogue 3: out (float32) = D. bias may be NULL, and may start at any float. */
 wm_status wm_op_linear(const void* A, const void* W, const float* bias, void* out, int M, int N, int K,
                        int precision, int epilogue, void* stream);
 
@@ -371,13 +380,19 @@ wm_status wm_set_fused_mlp(int enable);
  * Appendix A.2 blocks): 1 (the default) lets wm_latent_rollout and
  * wm_rollout_batch run BF16 contexts with C = 128, 4 heads, periodic
  * longitude, no rotary embedding, H % 8 == 0, W % 16 == 0, W >= 32 and
- * latitude / longitude windows of at most 5 as ONE kernel launch per group of
- * latents (as many as the device holds at once: 4 for the 4 x 24 x 48 latent).
+ * latitude / longitude windows of at most 5 as kernel launches over whole
+ * rollouts, each for as many latents as the device holds at once (4 for the
+ * 4 x 24 x 48 latent); wm_rollout_batch cuts uneven rollouts at steps into more
+ * launches where that keeps them filled.
  * Each CTA keeps an 8 x 16-token patch (8 x 8 or 8 x 4 where few latents share
  * the launch; same results) of its latent's residual stream in
- * shared memory for the whole rollout and runs every block's attention,
+ * tensor memory for the whole launch and runs every block's attention,
  * projection, MLP, LayerNorms and residual adds; the latent's CTAs meet once
- * per block at a counter in global memory. The result equals the per-kernel
+ * per block at a counter in global memory. The patch follows from the latents
+ * of the launch and from the streams of this process lately seen with such
+ * launches in flight on the device; a launch captured by the caller keeps the
+ * patch of its capture, which leaves room for one launch of every context that
+ * then holds the kernel. The result equals the per-kernel
  * path within the BF16 tolerance (LayerNorm is applied explicitly, not folded
  * into the GEMMs, so the two are not bit-identical). Latents of
  * wm_rollout_batch are read and written in place. 0: every rollout uses one
